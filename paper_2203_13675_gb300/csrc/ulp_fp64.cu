@@ -484,9 +484,13 @@ __device__ __forceinline__ void coef_tile(const PcgArgs& a, const MapDesc& M, in
 // earlier-ordered slot step has already been given (no cycle).
 template <int MODE>
 __device__ bool sweep_phase(const PcgArgs& a, const int* s_bbase, bool (*want)(const MapState*)) {
-  const int lane = threadIdx.x & 31;
-  const int slot = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-  const int NS = gridDim.x * kWarps;
+  extern __shared__ __align__(16) unsigned char sweep_dsm[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int pair = warp % kSweepPairs;
+  const bool helper = warp >= kSweepPairs;
+  SweepSmem& sm = reinterpret_cast<SweepSmem*>(sweep_dsm)[pair];
+  const int slot = pair * gridDim.x + blockIdx.x;
+  const int NS = gridDim.x * kSweepPairs;
   for (int k = slot; k < a.nbands; k += NS) {
     const int gb = (MODE == kSweepBwd) ? a.nbands - 1 - k : k;
     const int m = find_map(s_bbase, a.nmaps, gb);
@@ -506,8 +510,9 @@ __device__ bool sweep_phase(const PcgArgs& a, const int* s_bbase, bool (*want)(c
       if (band > 0) io.xin = M.xf + (size_t)(band - 1) * P;
       if (band + 1 < nb) io.xout = M.xf + (size_t)band * P;
     }
-    if (!band_sweep<MODE>(M, band, lane, io, a.timeout_ns, &a.bar->err))
-      return false;  // the error flag is set: the next grid barrier ends every block
+    const bool ok = helper ? sweep_helper<MODE>(M, band, lane, io, sm, pair, a.timeout_ns, &a.bar->err)
+                           : sweep_compute<MODE>(M, band, lane, io, sm, pair);
+    if (!ok) return false;  // the error flag is set: the next grid barrier ends every block
   }
   return true;
 }
@@ -855,9 +860,17 @@ int pcg64_max_blocks_per_sm(int kind) {
   switch (kind) {
     case kIdentity: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pcg64<kIdentity>, kThreads, 0); break;
     case kJacobi: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pcg64<kJacobi>, kThreads, 0); break;
+    // dynamic shared memory above 48 KB is an attribute of the function on the current
+    // device: set here, which every plan creation passes
     case kIlu:
-    case kIc: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pcg64_sweep<kIlu>, kThreads, 0); break;
-    case kSsor: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pcg64_sweep<kSsor>, kThreads, 0); break;
+    case kIc:
+      cudaFuncSetAttribute(k_pcg64_sweep<kIlu>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmem);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pcg64_sweep<kIlu>, kThreads, kSweepSmem);
+      break;
+    case kSsor:
+      cudaFuncSetAttribute(k_pcg64_sweep<kSsor>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmem);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pcg64_sweep<kSsor>, kThreads, kSweepSmem);
+      break;
     default: nb = 0;
   }
   return nb;
@@ -882,12 +895,12 @@ cudaError_t launch_pcg64(const Plan& pl, int kind, const PcgArgs& a, cudaStream_
     case kIlu:
     case kIc: {
       void* args[] = {(void*)&a};
-      e = cudaLaunchCooperativeKernel((void*)k_pcg64_sweep<kIlu>, pl.nsm * pl.bps_sweep, kThreads, args, 0, st);
+      e = cudaLaunchCooperativeKernel((void*)k_pcg64_sweep<kIlu>, pl.nsm * pl.bps_sweep, kThreads, args, kSweepSmem, st);
       break;
     }
     case kSsor: {
       void* args[] = {(void*)&a};
-      e = cudaLaunchCooperativeKernel((void*)k_pcg64_sweep<kSsor>, pl.nsm * pl.bps_sweep, kThreads, args, 0, st);
+      e = cudaLaunchCooperativeKernel((void*)k_pcg64_sweep<kSsor>, pl.nsm * pl.bps_sweep, kThreads, args, kSweepSmem, st);
       break;
     }
     default: e = cudaErrorInvalidValue;
