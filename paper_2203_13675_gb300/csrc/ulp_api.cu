@@ -117,6 +117,7 @@ void ulp::phase_mark(Plan& pl, cudaStream_t st, int tag) {
 // solver (static round-robin assignment, so equal counts balance the work),
 // between 4 and 64 rows so the two halo rows stay amortised.
 int ulp::solver_blocks_per_sm() {
+  resident_attrs();
   int occ = 1 << 30;
   for (int kind : {kIdentity, kJacobi}) {
     const int o = pcg64_max_blocks_per_sm(kind), o2 = pcg32_max_blocks_per_sm(kind);
@@ -203,6 +204,9 @@ static int plan_init(Plan& pl, int n, const int* H, const int* W, const ulp_opti
   bytes += align256(sizeof(MapStats) * n);
   const size_t off_part = bytes;
   bytes += 3 * align256(sizeof(double) * tiles);
+  const size_t off_flow = bytes;
+  pl.nflow = tiles > pl.nsm + n ? tiles : pl.nsm + n;
+  bytes += align256(sizeof(double) * kFlowSlots * pl.nflow);
   const size_t off_outer = bytes;
   bytes += align256(sizeof(double) * 2 * (size_t)n * pl.bx_elem);
   const size_t off_bar = bytes;
@@ -245,6 +249,7 @@ static int plan_init(Plan& pl, int n, const int* H, const int* W, const ulp_opti
   pl.P0 = reinterpret_cast<double*>(base + off_part);
   pl.P1 = reinterpret_cast<double*>(base + off_part + align256(sizeof(double) * tiles));
   pl.P2 = reinterpret_cast<double*>(base + off_part + 2 * align256(sizeof(double) * tiles));
+  pl.flow = reinterpret_cast<double*>(base + off_flow);
   pl.outer_part = reinterpret_cast<double*>(base + off_outer);
   pl.bar = reinterpret_cast<Barrier*>(base + off_bar);
   pl.n_active = reinterpret_cast<int*>(base + off_bar + align256(sizeof(Barrier)));
@@ -351,6 +356,8 @@ static PcgArgs pcg_args(const Plan& pl, double tol, int max_inner) {
   a.P0 = pl.P0;
   a.P1 = pl.P1;
   a.P2 = pl.P2;
+  a.flow = pl.flow;
+  a.nflow = pl.nflow;
   a.bar = pl.bar;
   a.n_active = pl.n_active;
   a.stop_mode = pl.opt.stop_mode;

@@ -455,16 +455,16 @@ __device__ __forceinline__ void warp_arrive_fcg(const PcgArgs& a, const MapDesc&
   }
 }
 
-// d = s + beta d_old, q = A d, partial d^T q (Algorithm 1: q <- A d, d^T q).
+// d = s + beta d_old, q = A d on one tile; the lane's share of d^T q (Algorithm 1: q <- A d, d^T q).
 template <int KIND>
-__device__ __forceinline__ void a_tile(const PcgArgs& a, const MapDesc& M, MapState* S, int t, int lane) {
+__device__ __forceinline__ double a_tile_dq(const PcgArgs& a, const MapDesc& M, int t, long long it, double beta,
+                                            int lane) {
   const TileGeo g = tile_geo(M, t, a.R);
   const size_t P = M.pitch;
-  const long long it = *(volatile long long*)&S->iter;
   const double* sv = (KIND == kIdentity) ? M.f.r : M.f.s;
   const double* dold = (it & 1) ? M.f.d1 : M.f.d0;
   double* dnew = (it & 1) ? M.f.d0 : M.f.d1;
-  XDir x{sv, dold, *(volatile double*)&S->beta, it == 0, P};
+  XDir x{sv, dold, beta, it == 0, P};
   double dq = 0.0;
   auto epi = [&](size_t off, double2 xc, double2 ax) {
     st2(dnew, off, xc);
@@ -473,6 +473,12 @@ __device__ __forceinline__ void a_tile(const PcgArgs& a, const MapDesc& M, MapSt
     dq = fma(xc.y, ax.y, dq);
   };
   stencil_tile(M, g.i0, g.i1, g.j0, lane, M.f.U, M.f.V, M.f.D, x, epi);
+  return dq;
+}
+// The same as phase A of a solve whose scalars live in the map's state.
+template <int KIND>
+__device__ __forceinline__ void a_tile(const PcgArgs& a, const MapDesc& M, MapState* S, int t, int lane) {
+  const double dq = a_tile_dq<KIND>(a, M, t, *(volatile long long*)&S->iter, *(volatile double*)&S->beta, lane);
   tile_arrive(a, M, S, t, kPhA, dq, 0.0, 0.0, lane);
 }
 

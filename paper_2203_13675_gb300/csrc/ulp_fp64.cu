@@ -6,6 +6,7 @@
 #include "ulp_host.h"
 #include "ulp_sweep.cuh"
 #include "ulp_engine.cuh"
+#include "ulp_flow.cuh"
 
 #include <math.h>
 
@@ -218,47 +219,16 @@ __global__ void k_system_x(const MapDesc* __restrict__ maps, MapState* S) {
   }
 }
 
-// r = b - A phi, s = M^{-1} r, partials r^T s, r^T r (and b^T b at the start).
-template <int KIND>
-__device__ __forceinline__ void res_tile(const PcgArgs& a, const MapDesc& M, MapState* S, int t,
-                                         bool init, int lane) {
-  const TileGeo g = tile_geo(M, t, a.R);
-  const size_t P = M.pitch;
-  XPlane x{M.f.phi, P};
-  double rs = 0.0, rr = 0.0, bb = 0.0;
-  auto epi = [&](size_t off, double2 xc, double2 ax) {
-    const double2 bv = ld2(M.f.b, off);
-    double2 r = make_double2(bv.x - ax.x, bv.y - ax.y);
-    st2(M.f.r, off, r);
-    if (KIND == kJacobi) {
-      const double2 di = ld2(M.f.Dinv, off);
-      const double2 s = make_double2(di.x * r.x, di.y * r.y);
-      st2(M.f.s, off, s);
-      rs = fma(r.x, s.x, rs);
-      rs = fma(r.y, s.y, rs);
-    }
-    rr = fma(r.x, r.x, rr);
-    rr = fma(r.y, r.y, rr);
-    if (init) {
-      bb = fma(bv.x, bv.x, bb);
-      bb = fma(bv.y, bv.y, bb);
-    }
-  };
-  stencil_tile(M, g.i0, g.i1, g.j0, lane, M.f.U, M.f.V, M.f.D, x, epi);
-  if (KIND == kIdentity) rs = rr;
-  tile_arrive(a, M, S, t, init ? kPhResInit : kPhRes, rs, rr, bb, lane);
-}
-
 // phi += alpha d; r -= alpha q; s = M^{-1} r; partials r^T s, r^T r.
 // On a refresh iteration only phi is updated (the residual is recomputed).
 template <int KIND>
-__device__ __forceinline__ void b_tile(const PcgArgs& a, const MapDesc& M, MapState* S, int t,
-                                       bool refresh, int lane) {
+__device__ __forceinline__ void b_tile(const PcgArgs& a, const MapDesc& M, const FlowMap& L, int t, int lane) {
   const TileGeo g = tile_geo(M, t, a.R);
   const size_t P = M.pitch;
-  const long long it = *(volatile long long*)&S->iter;
+  const long long it = L.iter;
+  const bool refresh = (it % M.refresh) == 0;
   const double* d = (it & 1) ? M.f.d0 : M.f.d1;
-  const double alpha = *(volatile double*)&S->alpha;
+  const double alpha = L.alpha;
   const int j = g.j0 + 2 * lane;
   const double2 z2 = make_double2(0.0, 0.0);
   double rs = 0.0, rr = 0.0;
@@ -308,66 +278,44 @@ __device__ __forceinline__ void b_tile(const PcgArgs& a, const MapDesc& M, MapSt
   }
   if (!refresh) {
     if (KIND == kIdentity) rs = rr;
-    tile_arrive(a, M, S, t, kPhB, rs, rr, 0.0, lane);
+    rs = warp_sum(rs);
+    rr = warp_sum(rr);
   }
+  flow_publish(a, L, t, rs, rr, 0.0, lane);
 }
 
 // The inner PCG of Algorithm 1 for every map of the call, as one persistent
-// cooperative kernel: phases separated by grid barriers, per-map scalars
-// advanced by the last warp of each phase.  Maps that converge drop out.
+// cooperative kernel: every map goes through its phases (start, A, B, on refresh
+// iterations the true residual) at its own pace, its scalars advanced by every block
+// that owns tiles of it (ulp_flow.cuh).
 template <int KIND>
 __global__ void __launch_bounds__(kThreads, 2) k_pcg64(PcgArgs a) {
-  __shared__ int s_base[kMaxMaps + 1];
-  __shared__ int s_any;
-  for (int m = threadIdx.x; m <= a.nmaps; m += blockDim.x)
-    s_base[m] = (m < a.nmaps) ? a.maps[m].tile_base : a.ntiles;
-  __syncthreads();
+  __shared__ FlowShared fs;
   const int lane = threadIdx.x & 31;
   const int gw = blockIdx.x * kWarps + (threadIdx.x >> 5);
   const int NW = gridDim.x * kWarps;
-
-  for (int t = gw; t < a.ntiles; t += NW) {
-    const int m = find_map(s_base, a.nmaps, t);
-    MapState* S = a.st + m;
-    if (*(volatile int*)&S->done) continue;
-    res_tile<KIND>(a, a.maps[m], S, t, true, lane);
-  }
-  if (!grid_sync(a.bar, a.timeout_ns)) return;
-
-  for (int g = 0;; ++g) {
-    if (*(volatile int*)a.n_active == 0) break;
+  flow_begin(a, fs, blockIdx.x * kWarps, kWarps, NW);
+  while (fs.alive > 0) {
     for (int t = gw; t < a.ntiles; t += NW) {
-      const int m = find_map(s_base, a.nmaps, t);
-      MapState* S = a.st + m;
-      if (*(volatile int*)&S->done) continue;
-      a_tile<KIND>(a, a.maps[m], S, t, lane);
-    }
-    if (!grid_sync(a.bar, a.timeout_ns)) return;
-    // refresh iterations (l mod period = 0) are a static function of g
-    if (threadIdx.x == 0) s_any = 0;
-    __syncthreads();
-    for (int m = threadIdx.x; m < a.nmaps; m += blockDim.x)
-      if (g % a.maps[m].refresh == 0) s_any = 1;
-    __syncthreads();
-    const bool any_refresh = s_any != 0;
-    for (int t = gw; t < a.ntiles; t += NW) {
-      const int m = find_map(s_base, a.nmaps, t);
-      MapState* S = a.st + m;
-      if (*(volatile int*)&S->done) continue;
+      const int m = find_map(fs.base, a.nmaps, t);
+      const FlowMap& L = fs.loc[fs.slot[m]];
+      if (L.done) continue;
       const MapDesc& M = a.maps[m];
-      b_tile<KIND>(a, M, S, t, (g % M.refresh) == 0, lane);
-    }
-    if (!grid_sync(a.bar, a.timeout_ns)) return;
-    if (any_refresh) {
-      for (int t = gw; t < a.ntiles; t += NW) {
-        const int m = find_map(s_base, a.nmaps, t);
-        MapState* S = a.st + m;
-        const MapDesc& M = a.maps[m];
-        if (*(volatile int*)&S->done || (g % M.refresh) != 0) continue;
-        res_tile<KIND>(a, M, S, t, false, lane);
+      if (L.phase == kPhA) {
+        const double dq = warp_sum(a_tile_dq<KIND>(a, M, t, L.iter, L.beta, lane));
+        flow_publish(a, L, t, dq, 0.0, 0.0, lane);
+      } else if (L.phase == kPhB) {
+        b_tile<KIND>(a, M, L, t, lane);
+      } else {
+        double rs, rr, bb;
+        res_tile<KIND>(a, M, L.phase == kPhResInit, t, lane, rs, rr, bb);
+        rs = warp_sum(rs);
+        rr = warp_sum(rr);
+        if (L.phase == kPhResInit) bb = warp_sum(bb);
+        flow_publish(a, L, t, rs, rr, bb, lane);
       }
-      if (!grid_sync(a.bar, a.timeout_ns)) return;
     }
+    if (!flow_step(a, fs)) return;
   }
 }
 
@@ -610,8 +558,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_pcg64_sweep(PcgArgs a) {
   }
 }
 
-// Resets the per-map solver state before a PCG launch.
-__global__ void k_pcg_reset(MapState* S, int nmaps, int* n_active, Barrier* bar) {
+// Resets the per-map solver state before a PCG launch (block 0) and fills the persistent
+// kernels' slots with the sentinel (the other blocks).
+__global__ void k_pcg_reset(MapState* S, int nmaps, int* n_active, Barrier* bar, double* flow, size_t nflow) {
+  if (blockIdx.x > 0) {
+    for (size_t k = (blockIdx.x - 1) * (size_t)blockDim.x + threadIdx.x; k < nflow; k += (size_t)(gridDim.x - 1) * blockDim.x)
+      st_relaxed(flow + k, sentinel());
+    return;
+  }
   __shared__ int s_cnt;
   if (threadIdx.x == 0) s_cnt = 0;
   __syncthreads();
@@ -876,22 +830,29 @@ int pcg64_max_blocks_per_sm(int kind) {
   return nb;
 }
 
-void launch_pcg_reset(const Plan& pl, cudaStream_t st) {
-  k_pcg_reset<<<1, kThreads, 0, st>>>(pl.dstate, pl.nmaps, pl.n_active, pl.bar);
+void launch_pcg_reset(const Plan& pl, cudaStream_t st, bool flow) {
+  const size_t n = flow ? (size_t)kFlowSlots * pl.nflow : 0;
+  const size_t nb = (n + 4 * kThreads - 1) / (4 * kThreads);
+  k_pcg_reset<<<1 + (int)(nb < (size_t)pl.nsm ? nb : pl.nsm), kThreads, 0, st>>>(pl.dstate, pl.nmaps, pl.n_active,
+                                                                               pl.bar, pl.flow, n);
 }
 
 cudaError_t launch_pcg64(const Plan& pl, int kind, const PcgArgs& a, cudaStream_t st, cudaEvent_t e0,
                          cudaEvent_t e1) {
   pl.kernel_launches += 2;
   pl.solver_launches += 1;
-  k_pcg_reset<<<1, kThreads, 0, st>>>(pl.dstate, pl.nmaps, pl.n_active, pl.bar);
+  launch_pcg_reset(pl, st, kind == kIdentity || kind == kJacobi);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (e0) cudaEventRecord(e0, st);
   const int blocks = pl.nsm * pl.bps;
   switch (kind) {
-    case kIdentity: e = launch_pcg64_kind<kIdentity>(pl, a, blocks, st); break;
-    case kJacobi: e = launch_pcg64_kind<kJacobi>(pl, a, blocks, st); break;
+    case kIdentity:
+    case kJacobi:
+      if (resident_fits(pl, true, kind)) e = launch_resident(pl, true, kind, a, st);
+      else if (kind == kIdentity) e = launch_pcg64_kind<kIdentity>(pl, a, blocks, st);
+      else e = launch_pcg64_kind<kJacobi>(pl, a, blocks, st);
+      break;
     case kIlu:
     case kIc: {
       void* args[] = {(void*)&a};

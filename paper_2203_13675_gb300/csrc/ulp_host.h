@@ -29,6 +29,8 @@ struct Plan {
   MapState* dstate = nullptr;
   MapStats* dstats = nullptr;
   double *P0 = nullptr, *P1 = nullptr, *P2 = nullptr;
+  double* flow = nullptr;    // kFlowSlots arrays of nflow slots: per tile, or per block and map
+  int nflow = 0;
   double* outer_part = nullptr;
   Barrier* bar = nullptr;
   int* n_active = nullptr;
@@ -98,7 +100,8 @@ cudaError_t launch_outer_error(const Plan& pl, double outer_tol, int max_outer, 
 cudaError_t launch_pcg64(const Plan& pl, int kind, const PcgArgs& a, cudaStream_t st, cudaEvent_t e0 = nullptr,
                          cudaEvent_t e1 = nullptr);
 int pcg64_max_blocks_per_sm(int kind);
-void launch_pcg_reset(const Plan& pl, cudaStream_t st);
+// flow: also the slots of the persistent kernels' published partials
+void launch_pcg_reset(const Plan& pl, cudaStream_t st, bool flow = false);
 
 // ulp_dct.cu
 size_t dct_bytes(int H, int W);
@@ -164,6 +167,12 @@ int matvec_on_plan(ulp_plan plan, const double* U, const double* V, const double
 cudaError_t launch_fcg(Plan& pl, int kind, const PcgArgs& a, cudaStream_t st, cudaEvent_t e0 = nullptr,
                        cudaEvent_t e1 = nullptr);
 void destroy_fcg(Plan& pl);
+
+// ulp_resident.cu: the Jacobi / identity solvers with their working set on the chip; whether
+// the plan's tiles fit, and the launch (attributes are set on the current device first)
+void resident_attrs();
+bool resident_fits(const Plan& pl, bool f64, int kind);
+cudaError_t launch_resident(const Plan& pl, bool f64, int kind, const PcgArgs& a, cudaStream_t st);
 
 // ulp_mixed.cu
 cudaError_t launch_pcg32(const Plan& pl, int kind, const PcgArgs& a, cudaStream_t st, cudaEvent_t e0 = nullptr,

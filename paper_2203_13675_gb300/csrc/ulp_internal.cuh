@@ -111,6 +111,8 @@ struct PcgArgs {
   MapState* st;
   int nmaps, ntiles, R, nbands;
   double *P0, *P1, *P2;     // per-tile partial sums
+  double* flow;             // persistent PCG: slots of the published partials, kFlowSlots arrays
+  int nflow;                // of this many (a slot per tile, or per block and map)
   Barrier* bar;
   int* n_active;
   int stop_mode;
@@ -130,6 +132,10 @@ struct PcgArgs {
   int xfcg;                 // mixed flexible CG: convergence of the FP32 recurrence is confirmed on the
                             // FP64 true residual before the solve stops
 };
+
+// Arrays of slots of the persistent PCG kernels' published partials: three sets of two sums
+// (four in the resident kernels), and b^T b at the start.
+constexpr int kFlowSlots = 9;
 
 // ------------------------------------------------------------------ helpers
 __device__ __forceinline__ unsigned long long globaltimer() {

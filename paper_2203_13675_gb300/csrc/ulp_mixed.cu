@@ -13,62 +13,10 @@
 //     step, every 20 iterations here) the FP32 correction is folded into phi
 //     and r = b - A phi is recomputed with the FP64 weights and FP64 phi.
 // Bytes per pixel per iteration: 24 (phase A) + 32 (phase B) versus 112 in FP64.
-#include "ulp_mixed.cuh"
+#include "ulp_flow32.cuh"
 #include "ulp_host.h"
 
 namespace ulp {
-
-// FP32 copies of the weights and the Jacobi inverse; the correction starts at 0.
-template <int KIND>
-__device__ __forceinline__ void conv_tile(const PcgArgs& a, const MapDesc& M, int t, int lane) {
-  const TileGeo g = tile_geo(M, t, a.R);
-  const size_t P = M.pitch;
-  const int j = g.j0 + 2 * lane;
-  for (int i = g.i0; i < g.i1; ++i) {
-    const size_t off = (size_t)i * P + j;
-    const double2 u = ld2(M.f.U, off), v = ld2(M.f.V, off);
-    stf2(M.h.U, off, make_float2((float)u.x, (float)u.y));
-    stf2(M.h.V, off, make_float2((float)v.x, (float)v.y));
-    if (KIND == kJacobi) {
-      const double2 di = ld2(M.f.Dinv, off);
-      stf2(M.h.Dinv, off, make_float2((float)di.x, (float)di.y));
-    }
-    stf2(M.h.x, off, make_float2(0.f, 0.f));
-  }
-}
-
-// True residual in FP64: r = b - A phi (FP64 weights, FP64 phi), rounded to
-// FP32 for the recurrence; s = M^-1 r; partials r^T s, r^T r (and b^T b).
-template <int KIND>
-__device__ __forceinline__ void res64_tile(const PcgArgs& a, const MapDesc& M, MapState* S, int t, bool init,
-                                           int lane) {
-  const TileGeo g = tile_geo(M, t, a.R);
-  XPlane x{M.f.phi, (size_t)M.pitch};
-  DF rs, rr;
-  double bb = 0.0;
-  auto epi = [&](size_t off, double2, double2 ax) {
-    const double2 bv = ld2(M.f.b, off);
-    const float2 r = make_float2((float)(bv.x - ax.x), (float)(bv.y - ax.y));
-    stf2(M.h.r, off, r);
-    if (KIND == kJacobi) {
-      const float2 di = ldf2(M.h.Dinv, off);
-      const float2 s = make_float2(di.x * r.x, di.y * r.y);
-      stf2(M.h.s, off, s);
-      rs.add_prod(r.x, s.x);
-      rs.add_prod(r.y, s.y);
-    }
-    rr.add_prod(r.x, r.x);
-    rr.add_prod(r.y, r.y);
-    if (init) {
-      bb = fma(bv.x, bv.x, bb);
-      bb = fma(bv.y, bv.y, bb);
-    }
-  };
-  stencil_tile(M, g.i0, g.i1, g.j0, lane, M.f.U, M.f.V, M.f.D, x, epi);
-  const double vrr = rr.value();
-  const double vrs = (KIND == kIdentity) ? vrr : rs.value();
-  tile_arrive(a, M, S, t, init ? kPhResInit : kPhRes, vrs, vrr, bb, lane);
-}
 
 // Phase B's ring slots (kRingB32 per warp, inside the warp's share of phase A's ring).
 constexpr int kLeadB32 = 3;
@@ -83,13 +31,14 @@ static_assert(kRingB32 * sizeof(SlotB32) <= kRing32 * sizeof(Slot32), "phase B's
 // wring: the warp's share of phase A's ring, through which the rows stream kLeadB32
 // ahead (or null, and on refresh iterations: loads two rows ahead in registers).
 template <int KIND>
-__device__ __forceinline__ void b32_tile(const PcgArgs& a, const MapDesc& M, MapState* S, int t, bool refresh,
-                                         int lane, unsigned char* wring) {
+__device__ __forceinline__ void b32_tile(const PcgArgs& a, const MapDesc& M, const FlowMap& L, int t, int lane,
+                                         unsigned char* wring) {
   const TileGeo g = tile_geo(M, t, a.R);
   const size_t P = M.pitch;
-  const long long it = *(volatile long long*)&S->iter;
+  const long long it = L.iter;
+  const bool refresh = (it % M.refresh) == 0;
   const float* d = (it & 1) ? M.h.d0 : M.h.d1;
-  const float alpha = (float)*(volatile double*)&S->alpha;
+  const float alpha = (float)L.alpha;
   const int j = g.j0 + 2 * lane;
   const float2 z2 = make_float2(0.f, 0.f);
   struct Row {
@@ -153,7 +102,7 @@ __device__ __forceinline__ void b32_tile(const PcgArgs& a, const MapDesc& M, Map
     }
     cpa_wait_all();
     const double vrr = rr.value();
-    tile_arrive(a, M, S, t, kPhB, (KIND == kIdentity) ? vrr : rs.value(), vrr, 0.0, lane);
+    flow_publish(a, L, t, warp_sum((KIND == kIdentity) ? vrr : rs.value()), warp_sum(vrr), 0.0, lane);
     return;
   }
   Row c0 = load(g.i0), c1 = load(g.i0 + 1);
@@ -187,10 +136,9 @@ __device__ __forceinline__ void b32_tile(const PcgArgs& a, const MapDesc& M, Map
     c0 = c1;
     c1 = c2;
   }
-  if (!refresh) {
-    const double vrr = rr.value();
-    tile_arrive(a, M, S, t, kPhB, (KIND == kIdentity) ? vrr : rs.value(), vrr, 0.0, lane);
-  }
+  const double vrr = rr.value();
+  flow_publish(a, L, t, refresh ? 0.0 : warp_sum((KIND == kIdentity) ? vrr : rs.value()), refresh ? 0.0 : warp_sum(vrr),
+               0.0, lane);
 }
 
 // phi += x, x = 0 (end of the solve).
@@ -209,67 +157,61 @@ __device__ __forceinline__ void fold_tile(const PcgArgs& a, const MapDesc& M, in
   }
 }
 
+// phase A's row rings, phase B's in turn (dynamic: they share the block with FlowShared)
+struct Rings32 {
+  Slot32 s[kWarps][kRing32];
+};
+
+// The whole inner solve of every map, as k_pcg64.
 template <int KIND>
 __global__ void __launch_bounds__(kThreads, 2) k_pcg32(PcgArgs a) {
-  __shared__ Slot32 ring32[kWarps][kRing32];  // phase A's row rings, phase B's in turn
-  __shared__ int s_base[kMaxMaps + 1];
-  __shared__ int s_any;
-  for (int m = threadIdx.x; m <= a.nmaps; m += blockDim.x)
-    s_base[m] = (m < a.nmaps) ? a.maps[m].tile_base : a.ntiles;
-  __syncthreads();
+  extern __shared__ __align__(16) unsigned char pcg32_dsm[];
+  Slot32* ring = reinterpret_cast<Rings32*>(pcg32_dsm)->s[threadIdx.x >> 5];
+  __shared__ FlowShared fs;
   const int lane = threadIdx.x & 31;
   const int gw = blockIdx.x * kWarps + (threadIdx.x >> 5);
   const int NW = gridDim.x * kWarps;
-  auto for_tiles = [&](auto&& body) {
+  flow_begin(a, fs, blockIdx.x * kWarps, kWarps, NW);
+  while (fs.alive > 0) {
     for (int t = gw; t < a.ntiles; t += NW) {
-      const int m = find_map(s_base, a.nmaps, t);
-      MapState* S = a.st + m;
-      if (*(volatile int*)&S->done) continue;
-      body(a.maps[m], S, t);
+      const int m = find_map(fs.base, a.nmaps, t);
+      const FlowMap& L = fs.loc[fs.slot[m]];
+      if (L.done) continue;
+      const MapDesc& M = a.maps[m];
+      if (L.phase == kPhA) {
+        const double dq = warp_sum(a32_tile_dq<KIND>(a, M, t, L.iter, L.beta, lane, ring));
+        flow_publish(a, L, t, dq, 0.0, 0.0, lane);
+      } else if (L.phase == kPhB) {
+        b32_tile<KIND>(a, M, L, t, lane, reinterpret_cast<unsigned char*>(ring));
+      } else {
+        // the start: the tile's FP32 planes first (the residual reads only its own pixels of them)
+        if (L.phase == kPhResInit) conv_tile<KIND>(a, M, t, lane);
+        const bool init = L.phase == kPhResInit;
+        double rs, rr, bb;
+        res64_tile<KIND>(a, M, init, t, lane, rs, rr, bb);
+        flow_publish(a, L, t, warp_sum(rs), warp_sum(rr), init ? warp_sum(bb) : 0.0, lane);
+      }
     }
-  };
-  // maps active at the start: the final fold must reach them after they stop
-  auto for_tiles_started = [&](auto&& body) {
-    for (int t = gw; t < a.ntiles; t += NW) {
-      const int m = find_map(s_base, a.nmaps, t);
-      if (!a.st[m].outer_active) continue;
-      body(a.maps[m], t);
-    }
-  };
-
-  for_tiles([&](const MapDesc& M, MapState*, int t) { conv_tile<KIND>(a, M, t, lane); });
-  if (!grid_sync(a.bar, a.timeout_ns)) return;
-  for_tiles([&](const MapDesc& M, MapState* S, int t) { res64_tile<KIND>(a, M, S, t, true, lane); });
-  if (!grid_sync(a.bar, a.timeout_ns)) return;
-
-  for (int g = 0;; ++g) {
-    if (*(volatile int*)a.n_active == 0) break;
-    for_tiles([&](const MapDesc& M, MapState* S, int t) { a32_tile<KIND>(a, M, S, t, lane, ring32[threadIdx.x >> 5]); });
-    if (!grid_sync(a.bar, a.timeout_ns)) return;
-    if (threadIdx.x == 0) s_any = 0;
-    __syncthreads();
-    for (int m = threadIdx.x; m < a.nmaps; m += blockDim.x)
-      if (g % a.maps[m].refresh == 0) s_any = 1;
-    __syncthreads();
-    const bool any_refresh = s_any != 0;
-    for_tiles([&](const MapDesc& M, MapState* S, int t) {
-      b32_tile<KIND>(a, M, S, t, (g % M.refresh) == 0, lane, reinterpret_cast<unsigned char*>(ring32[threadIdx.x >> 5]));
-    });
-    if (!grid_sync(a.bar, a.timeout_ns)) return;
-    if (any_refresh) {
-      for_tiles([&](const MapDesc& M, MapState* S, int t) {
-        if ((g % M.refresh) == 0) res64_tile<KIND>(a, M, S, t, false, lane);
-      });
-      if (!grid_sync(a.bar, a.timeout_ns)) return;
-    }
+    if (!flow_step(a, fs)) return;
   }
-  for_tiles_started([&](const MapDesc& M, int t) { fold_tile(a, M, t, lane); });
+  // maps active at the start: what the correction holds goes into phi
+  for (int t = gw; t < a.ntiles; t += NW) {
+    const int m = find_map(fs.base, a.nmaps, t);
+    if (a.st[m].outer_active) fold_tile(a, a.maps[m], t, lane);
+  }
 }
 
 int pcg32_max_blocks_per_sm(int kind) {
   int nb = 0;
-  if (kind == kIdentity) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pcg32<kIdentity>, kThreads, 0);
-  else if (kind == kJacobi) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pcg32<kJacobi>, kThreads, 0);
+  // the attribute is the function's on the current device: set here, which every plan creation passes
+  const int smem = (int)sizeof(Rings32);
+  if (kind == kIdentity) {
+    cudaFuncSetAttribute(k_pcg32<kIdentity>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pcg32<kIdentity>, kThreads, smem);
+  } else if (kind == kJacobi) {
+    cudaFuncSetAttribute(k_pcg32<kJacobi>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pcg32<kJacobi>, kThreads, smem);
+  }
   return nb;
 }
 
@@ -277,16 +219,18 @@ cudaError_t launch_pcg32(const Plan& pl, int kind, const PcgArgs& a, cudaStream_
                          cudaEvent_t e1) {
   pl.kernel_launches += 2;
   pl.solver_launches += 1;
-  launch_pcg_reset(pl, st);
+  launch_pcg_reset(pl, st, true);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (e0) cudaEventRecord(e0, st);
   const int blocks = pl.nsm * pl.bps;
   void* args[] = {(void*)&a};
-  if (kind == kIdentity)
-    e = cudaLaunchCooperativeKernel((void*)k_pcg32<kIdentity>, blocks, kThreads, args, 0, st);
+  if (resident_fits(pl, false, kind))
+    e = launch_resident(pl, false, kind, a, st);
+  else if (kind == kIdentity)
+    e = cudaLaunchCooperativeKernel((void*)k_pcg32<kIdentity>, blocks, kThreads, args, sizeof(Rings32), st);
   else if (kind == kJacobi)
-    e = cudaLaunchCooperativeKernel((void*)k_pcg32<kJacobi>, blocks, kThreads, args, 0, st);
+    e = cudaLaunchCooperativeKernel((void*)k_pcg32<kJacobi>, blocks, kThreads, args, sizeof(Rings32), st);
   else
     e = cudaErrorInvalidValue;
   if (e == cudaSuccess && e1) e = cudaEventRecord(e1, st);

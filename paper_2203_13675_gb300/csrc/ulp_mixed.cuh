@@ -178,17 +178,16 @@ __device__ __forceinline__ void stencil_tile32(const MapDesc& M, int i0, int i1,
   cpa_wait_all();  // the next tile of this warp refills the same slots
 }
 
-// d = s + beta d_old, q = A d in FP32, d^T q FP64-accurate.
+// d = s + beta d_old, q = A d in FP32 on one tile; the lane's share of d^T q, FP64-accurate.
 // ring: the warp's kRing32 ring slots in shared memory
 template <int KIND>
-__device__ __forceinline__ void a32_tile(const PcgArgs& a, const MapDesc& M, MapState* S, int t, int lane,
-                                         Slot32* ring) {
+__device__ __forceinline__ double a32_tile_dq(const PcgArgs& a, const MapDesc& M, int t, long long it, double beta,
+                                              int lane, Slot32* ring) {
   const TileGeo g = tile_geo(M, t, a.R);
-  const long long it = *(volatile long long*)&S->iter;
   const float* sv = (KIND == kIdentity) ? M.h.r : M.h.s;
   const float* dold = (it & 1) ? M.h.d1 : M.h.d0;
   float* dnew = (it & 1) ? M.h.d0 : M.h.d1;
-  XDir32 x{sv, dold, (float)*(volatile double*)&S->beta, it == 0, (size_t)M.pitch};
+  XDir32 x{sv, dold, (float)beta, it == 0, (size_t)M.pitch};
   DF dq;
   auto epi = [&](size_t off, float2 xc, float2 ax) {
     stf2(dnew, off, xc);
@@ -197,7 +196,14 @@ __device__ __forceinline__ void a32_tile(const PcgArgs& a, const MapDesc& M, Map
     dq.add_prod(xc.y, ax.y);
   };
   stencil_tile32(M, g.i0, g.i1, g.j0, lane, M.h.U, M.h.V, x, epi, ring);
-  tile_arrive(a, M, S, t, kPhA, dq.value(), 0.0, 0.0, lane);
+  return dq.value();
+}
+// The same as phase A of a solve whose scalars live in the map's state.
+template <int KIND>
+__device__ __forceinline__ void a32_tile(const PcgArgs& a, const MapDesc& M, MapState* S, int t, int lane,
+                                         Slot32* ring) {
+  const double dq = a32_tile_dq<KIND>(a, M, t, *(volatile long long*)&S->iter, *(volatile double*)&S->beta, lane, ring);
+  tile_arrive(a, M, S, t, kPhA, dq, 0.0, 0.0, lane);
 }
 
 }  // namespace ulp

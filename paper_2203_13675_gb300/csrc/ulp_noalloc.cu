@@ -126,6 +126,8 @@ extern "C" int ulp_pcg_noalloc(const double* U, const double* V, const double* b
   pl.P0 = reinterpret_cast<double*>(p); p += a256(sizeof(double) * M.ntiles);
   pl.P1 = reinterpret_cast<double*>(p); p += a256(sizeof(double) * M.ntiles);
   pl.P2 = reinterpret_cast<double*>(p); p += a256(sizeof(double) * M.ntiles);
+  pl.nflow = M.ntiles > pl.nsm + 1 ? M.ntiles : pl.nsm + 1;
+  pl.flow = reinterpret_cast<double*>(p); p += a256(sizeof(double) * kFlowSlots * pl.nflow);
   pl.outer_part = reinterpret_cast<double*>(p); p += a256(sizeof(double) * 2 * pl.bx_elem);
   pl.bar = reinterpret_cast<Barrier*>(p); p += a256(sizeof(Barrier));
   pl.n_active = reinterpret_cast<int*>(p); p += a256(sizeof(int));
@@ -144,6 +146,8 @@ extern "C" int ulp_pcg_noalloc(const double* U, const double* V, const double* b
   a.P0 = pl.P0;
   a.P1 = pl.P1;
   a.P2 = pl.P2;
+  a.flow = pl.flow;
+  a.nflow = pl.nflow;
   a.bar = pl.bar;
   a.n_active = pl.n_active;
   a.stop_mode = ULP_STOP_RELRES;
