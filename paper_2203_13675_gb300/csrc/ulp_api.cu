@@ -202,8 +202,13 @@ static int plan_init(Plan& pl, int n, const int* H, const int* W, const ulp_opti
   bytes += align256(sizeof(MapState) * n);
   const size_t off_stats = bytes;
   bytes += align256(sizeof(MapStats) * n);
+  // partial sums per tile, or per unit of the mixed multigrid form's last kernel, whose units
+  // on small maps are more than the tiles (in FP64 the dot phase rides there only where they
+  // are not)
+  constexpr int kMgUnits = 2048;
+  const int npart = tiles > kMgUnits ? tiles : kMgUnits;
   const size_t off_part = bytes;
-  bytes += 3 * align256(sizeof(double) * tiles);
+  bytes += 3 * align256(sizeof(double) * npart);
   const size_t off_flow = bytes;
   pl.nflow = tiles > pl.nsm + n ? tiles : pl.nsm + n;
   bytes += align256(sizeof(double) * kFlowSlots * pl.nflow);
@@ -247,8 +252,8 @@ static int plan_init(Plan& pl, int n, const int* H, const int* W, const ulp_opti
   pl.dstate = reinterpret_cast<MapState*>(base + off_state);
   pl.dstats = reinterpret_cast<MapStats*>(base + off_stats);
   pl.P0 = reinterpret_cast<double*>(base + off_part);
-  pl.P1 = reinterpret_cast<double*>(base + off_part + align256(sizeof(double) * tiles));
-  pl.P2 = reinterpret_cast<double*>(base + off_part + 2 * align256(sizeof(double) * tiles));
+  pl.P1 = reinterpret_cast<double*>(base + off_part + align256(sizeof(double) * npart));
+  pl.P2 = reinterpret_cast<double*>(base + off_part + 2 * align256(sizeof(double) * npart));
   pl.flow = reinterpret_cast<double*>(base + off_flow);
   pl.outer_part = reinterpret_cast<double*>(base + off_outer);
   pl.bar = reinterpret_cast<Barrier*>(base + off_bar);
@@ -272,7 +277,8 @@ static int plan_init(Plan& pl, int n, const int* H, const int* W, const ulp_opti
       cudaGetLastError();
       return fail(ULP_ERR_NOMEM, "cudaMalloc(multigrid levels): %s", cudaGetErrorString(e));
     }
-    pl.mg = mg_create(pl.hmaps[0], pl.mg_mem, pl.nsm, pl.ntiles);
+    pl.mg = mg_create(pl.hmaps[0], pl.mg_mem, pl.nsm, pl.ntiles,
+                      pl.opt.precision == ULP_PRECISION_MIXED ? npart : pl.ntiles);
   }
   ULP_CU(cudaDeviceSynchronize());  // workspace zeroed before any stream may use it
   return ULP_OK;

@@ -139,54 +139,44 @@ __device__ __forceinline__ TileGeo tile_geo(const MapDesc& M, int t, int R) {
 // kPhConfirm: the true residual of a mixed flexible-CG confirmation body (its r^T r alone)
 enum Phase { kPhResInit = 0, kPhA = 1, kPhB = 2, kPhRes = 3, kPhFcg = 4, kPhConfirm = 5 };
 
-// Runs in the warp whose tile arrival completed phase `ph` for map m: reduces
-// the map's tile partials in a fixed order and advances its scalars
-// (alpha = delta_new / d^T q; delta_old, delta_new, beta; stop tests).
-// ngroups: how many group sums the arrival left (0: as many as the map's tiles make).
-// The finisher is the serial tail of its kernel (every other warp has left), so it is
-// built as few dependent memory round trips as possible: lane 0 loads every field of
-// the map's state it reads in the same round of L2 loads as the group sums (only the
-// finisher writes these fields, and every tile of the phase has arrived), works in
-// registers, and stores.  No fence closes it: the next phase reads the state after a
-// kernel boundary or after the grid barrier that follows every phase of the persistent
-// kernels (whose leading __syncthreads and fence cover this warp's stores).
-static_assert(kArriveGroups <= 32, "one lane per arrival group");
-__device__ __forceinline__ void finish_map(const PcgArgs& a, const MapDesc& M, MapState* Sp, int ph, int lane,
-                                           int ngroups = 0) {
+// The fields of a map's state that a phase's end reads, loaded as one round of L2 loads (by
+// the one thread that then advances them, as soon as nothing else changes them).
+struct ScalarIn {
+  double delta, delta0, bb, rr_best, rr_ref;
+  long long iter, loops;
+  int fallback, restart, stall, force_refresh, stop_after, confirm, refresh_next;
+};
+__device__ __forceinline__ ScalarIn load_scalars(const MapState* S) {
+  ScalarIn in;
+  in.delta = __ldcg(&S->delta);
+  in.delta0 = __ldcg(&S->delta0);
+  in.bb = __ldcg(&S->bb);
+  in.rr_best = __ldcg(&S->rr_best);
+  in.rr_ref = __ldcg(&S->rr_ref);
+  in.iter = __ldcg(&S->iter);
+  in.loops = __ldcg(&S->loops);
+  in.fallback = __ldcg(&S->fallback);
+  in.restart = __ldcg(&S->restart);
+  in.stall = __ldcg(&S->stall);
+  in.force_refresh = __ldcg(&S->force_refresh);
+  in.stop_after = __ldcg(&S->stop_after);
+  in.confirm = __ldcg(&S->confirm);
+  in.refresh_next = __ldcg(&S->refresh_next);
+  return in;
+}
+
+// Advances a map's scalars after phase ph from its sums (one thread); returns whether the map
+// is done.
+__device__ __forceinline__ bool finish_scalars(const PcgArgs& a, const MapDesc& M, MapState* Sp, const ScalarIn& in,
+                                               int ph, double v0, double v1, double v2) {
   volatile MapState* S = Sp;
-  // the per-group sums in group order, then a fixed shuffle tree
-  const int n = M.ntiles;
-  const int ng = ngroups > 0 ? ngroups : (n < kArriveGroups ? n : kArriveGroups);
-  const int cnt = (ph == kPhA) ? 1 : (ph == kPhResInit || ph == kPhFcg) ? 3 : 2;
-  const bool own = lane < ng;
-  // L2 loads: another warp wrote them, and this SM's L1 may hold an older phase's values
-  double v0 = own ? __ldcg(&Sp->gpart[0][lane]) : 0.0;
-  double v1 = (own && cnt > 1) ? __ldcg(&Sp->gpart[1][lane]) : 0.0;
-  double v2 = (own && cnt > 2) ? __ldcg(&Sp->gpart[2][lane]) : 0.0;
-  double delta = 0.0, delta0 = 0.0, bb = 0.0, rr_best = 0.0;
-  long long iter = 0;
-  int fallback = 0, restart = 0, stall = 0, force_refresh = 0, stop_after = 0, confirm = 0, refresh_next = 0;
-  double rr_ref = 0.0;
-  if (lane == 0) {
-    delta = __ldcg(&Sp->delta);
-    delta0 = __ldcg(&Sp->delta0);
-    bb = __ldcg(&Sp->bb);
-    rr_best = __ldcg(&Sp->rr_best);
-    iter = __ldcg(&Sp->iter);
-    fallback = __ldcg(&Sp->fallback);
-    restart = __ldcg(&Sp->restart);
-    stall = __ldcg(&Sp->stall);
-    force_refresh = __ldcg(&Sp->force_refresh);
-    stop_after = __ldcg(&Sp->stop_after);
-    confirm = __ldcg(&Sp->confirm);
-    refresh_next = __ldcg(&Sp->refresh_next);
-    rr_ref = __ldcg(&Sp->rr_ref);
-  }
-  v0 = warp_sum(v0);
-  v1 = cnt > 1 ? warp_sum(v1) : 0.0;
-  v2 = cnt > 2 ? warp_sum(v2) : 0.0;
+  double delta = in.delta, delta0 = in.delta0, bb = in.bb;
+  const double rr_best = in.rr_best, rr_ref = in.rr_ref;
+  long long iter = in.iter;
+  const int fallback = in.fallback, restart = in.restart, stall = in.stall, force_refresh = in.force_refresh,
+            stop_after = in.stop_after, confirm = in.confirm, refresh_next = in.refresh_next;
   bool done = false;
-  if (lane == 0) {
+  {
     bool refreshed = true;  // r is the true residual (mixed flexible CG: this iteration recomputed it)
     if (ph == kPhConfirm) {
       // the recurrence called the current iterate converged and this body recomputed its
@@ -284,7 +274,6 @@ __device__ __forceinline__ void finish_map(const PcgArgs& a, const MapDesc& M, M
       }
       const double tol2 = a.tol2;
       const bool conv = (a.stop_mode == 1) ? !(delta > tol2 * delta0) : !(rr > tol2 * bb);
-      S->relres = (bb > 0.0) ? sqrt(rr / bb) : 0.0;
       if (stop_after) {
         done = true;
       } else if (bb == 0.0 || conv) {
@@ -313,7 +302,43 @@ __device__ __forceinline__ void finish_map(const PcgArgs& a, const MapDesc& M, M
         done = true;
         S->status = 1;
       }
+      if (done) S->relres = (bb > 0.0) ? sqrt(rr / bb) : 0.0;  // read after the solve only
     }
+  }
+  return done;
+}
+
+// Runs in the warp whose tile arrival completed phase `ph` for map m: reduces
+// the map's tile partials in a fixed order and advances its scalars
+// (alpha = delta_new / d^T q; delta_old, delta_new, beta; stop tests).
+// ngroups: how many group sums the arrival left (0: as many as the map's tiles make).
+// The finisher is the serial tail of its kernel (every other warp has left), so it is
+// built as few dependent memory round trips as possible: lane 0 loads every field of
+// the map's state it reads in the same round of L2 loads as the group sums (only the
+// finisher writes these fields, and every tile of the phase has arrived), works in
+// registers, and stores.  No fence closes it: the next phase reads the state after a
+// kernel boundary or after the grid barrier that follows every phase of the persistent
+// kernels (whose leading __syncthreads and fence cover this warp's stores).
+static_assert(kArriveGroups <= 32, "one lane per arrival group");
+__device__ __forceinline__ void finish_map(const PcgArgs& a, const MapDesc& M, MapState* Sp, int ph, int lane,
+                                           int ngroups = 0) {
+  volatile MapState* S = Sp;
+  // the per-group sums in group order, then a fixed shuffle tree
+  const int n = M.ntiles;
+  const int ng = ngroups > 0 ? ngroups : (n < kArriveGroups ? n : kArriveGroups);
+  const int cnt = (ph == kPhA) ? 1 : (ph == kPhResInit || ph == kPhFcg) ? 3 : 2;
+  const bool own = lane < ng;
+  // L2 loads: another warp wrote them, and this SM's L1 may hold an older phase's values
+  double v0 = own ? __ldcg(&Sp->gpart[0][lane]) : 0.0;
+  double v1 = (own && cnt > 1) ? __ldcg(&Sp->gpart[1][lane]) : 0.0;
+  double v2 = (own && cnt > 2) ? __ldcg(&Sp->gpart[2][lane]) : 0.0;
+  const ScalarIn in = lane == 0 ? load_scalars(Sp) : ScalarIn{};
+  v0 = warp_sum(v0);
+  v1 = cnt > 1 ? warp_sum(v1) : 0.0;
+  v2 = cnt > 2 ? warp_sum(v2) : 0.0;
+  bool done = false;
+  if (lane == 0) {
+    done = finish_scalars(a, M, Sp, in, ph, v0, v1, v2);
     S->arrive = 0u;
   }
   // the arrival counters back to zero, one lane per group
@@ -394,65 +419,44 @@ __device__ __forceinline__ void tile_arrive(const PcgArgs& a, const MapDesc& M, 
   }
 }
 
-// Arrival of the flexible-CG dot phase from a kernel that covers the map with its
-// own decomposition into n warps (32 <= n <= the map's tile count), warp w: its
-// r^T s and r^T r go to P0, P1 at tile_base + w and count as above with n in
-// place of the tile count; the third sum's partials (r_{k+1}^T s_k left by phase B,
-// or b^T b at the start of a solve, ph = kPhResInit) are indexed by the map's
-// tiles, so the last warp of group g sums P2 over the map's tiles of group g.
-// Same fixed summation order on every run.
-// rr_tiles: r^T r comes, like the third sum, as per-tile partials in P1 (left by the
-// kernels that wrote r) instead of from this kernel.
-__device__ __forceinline__ void warp_arrive_fcg(const PcgArgs& a, const MapDesc& M, MapState* S, int w, int n,
-                                                double rs, double rr, int lane, int ph = kPhFcg,
-                                                bool rr_tiles = false) {
-  rs = warp_sum(rs);
-  if (!rr_tiles) rr = warp_sum(rr);
-  const int base = M.tile_base;
-  const int g = w % kArriveGroups;
-  const int gsize = (n - g + kArriveGroups - 1) / kArriveGroups;
-  const int gsize2 = g < M.ntiles ? (M.ntiles - g + kArriveGroups - 1) / kArriveGroups : 0;
-  int glast = 0;
-  if (lane == 0) {
-    __stcg(a.P0 + base + w, rs);
-    if (!rr_tiles) __stcg(a.P1 + base + w, rr);
-    glast = atom_add_acq_rel(&S->arrive_grp[g], 1u) == (unsigned)gsize - 1u;
-  }
-  glast = __shfl_sync(kFull, glast, 0);
-  if (!glast) return;
-  __syncwarp();
-  // one loop over both index ranges, so that all of a lane's loads are in flight together
-  // (each sum still runs over its own range in the same order)
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-  const int gmax = gsize > gsize2 ? gsize : gsize2;
-#pragma unroll 4
-  for (int m = lane; m < gmax; m += 32) {
-    const int idx = base + g + kArriveGroups * m;
-    if (m < gsize) {
-      s0 += __ldcg(a.P0 + idx);
-      if (!rr_tiles) s1 += __ldcg(a.P1 + idx);
+// Sum of one array of n partials by 128 threads (r = 0 .. 127), into part[32]: partial i
+// belongs to group i mod 32; within a group, lane l of 32 adds partials l, l + 32, ... of the
+// group in order and the lanes add up as a shuffle-down tree (16, 8, 4, 2, 1) -- tile_arrive's
+// order, so both give the same bits.  A thread holds lanes c, c + 4, ..., c + 28 of its group:
+// the tree's first three levels stay in registers, where an FP64 add of a warp costs its 64
+// cycles for 32 useful lanes instead of for a few.  get(i, v): loads v[q] = partial i + 128 q.
+struct GroupLane {
+  int g, c;
+  __device__ __forceinline__ explicit GroupLane(int r) : g(((r >> 5) << 3) + (r & 7)), c((r & 31) >> 3) {}
+  // first of the eight partials of round k (partial i + 4 kArriveGroups q for q = 0 .. 7)
+  __device__ __forceinline__ int first(int k) const { return g + kArriveGroups * (c + 32 * k); }
+};
+__device__ __forceinline__ void group_tree(const GroupLane& t, double (&acc)[8], double* part) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) acc[q] += acc[q + 4];
+  acc[0] += acc[2];
+  acc[1] += acc[3];
+  double s = acc[0] + acc[1];
+  s += __shfl_down_sync(kFull, s, 16);  // lanes c + 2 of the group
+  s += __shfl_down_sync(kFull, s, 8);   // lanes c + 1
+  if (t.c == 0) part[t.g] = s;
+}
+__device__ __forceinline__ void group_sums(const double* P, int n, int r, double* part) {
+  const GroupLane t(r);
+  double acc[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) acc[q] = 0.0;
+  for (int k = 0; t.first(k) < n; ++k) {
+    double v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int i = t.first(k) + 4 * kArriveGroups * q;
+      v[q] = i < n ? __ldcg(P + i) : 0.0;
     }
-    if (m < gsize2) {
-      s2 += __ldcg(a.P2 + idx);
-      if (rr_tiles) s1 += __ldcg(a.P1 + idx);
-    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc[q] += v[q];
   }
-  s0 = warp_sum(s0);
-  s1 = warp_sum(s1);
-  s2 = warp_sum(s2);
-  int last = 0;
-  if (lane == 0) {
-    volatile double* gp = &S->gpart[0][0];
-    gp[0 * kArriveGroups + g] = s0;
-    gp[1 * kArriveGroups + g] = s1;
-    gp[2 * kArriveGroups + g] = s2;
-    last = atom_add_acq_rel(&S->arrive, 1u) == (unsigned)kArriveGroups - 1u;
-  }
-  last = __shfl_sync(kFull, last, 0);
-  if (last) {
-    __syncwarp();
-    finish_map(a, M, S, ph, lane, kArriveGroups);
-  }
+  group_tree(t, acc, part);
 }
 
 // d = s + beta d_old, q = A d on one tile; the lane's share of d^T q (Algorithm 1: q <- A d, d^T q).
@@ -475,7 +479,7 @@ __device__ __forceinline__ double a_tile_dq(const PcgArgs& a, const MapDesc& M, 
   stencil_tile(M, g.i0, g.i1, g.j0, lane, M.f.U, M.f.V, M.f.D, x, epi);
   return dq;
 }
-// The same as phase A of a solve whose scalars live in the map's state.
+// The same as phase A of a solve whose scalars live in the map's state (arrival included).
 template <int KIND>
 __device__ __forceinline__ void a_tile(const PcgArgs& a, const MapDesc& M, MapState* S, int t, int lane) {
   const double dq = a_tile_dq<KIND>(a, M, t, *(volatile long long*)&S->iter, *(volatile double*)&S->beta, lane);

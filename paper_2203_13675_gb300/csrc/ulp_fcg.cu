@@ -26,6 +26,22 @@ namespace ulp {
 
 __global__ void k_set_args(PcgArgs a, PcgArgs* dst) { *dst = a; }
 
+// What the solve's kernels need of the plan, as a kernel parameter: the graph is captured
+// once per plan and kind, and read from device memory the descriptor cost every kernel two
+// dependent trips to L2 before its first load.  Only the tolerance and l_max change from call
+// to call; the kernels that test them take those from the arguments that k_set_args left.
+struct FcgArgs {
+  PcgArgs a;
+  MapDesc M;
+  const PcgArgs* call;
+};
+__device__ __forceinline__ PcgArgs call_args(const FcgArgs& f) {
+  PcgArgs a = f.a;
+  a.tol2 = __ldcg(&f.call->tol2);
+  a.lmax = __ldcg(&f.call->lmax);
+  return a;
+}
+
 // Set-up timing of a flexible-CG solve (plans with options.profile): end = 0 records the
 // start of the preconditioner's set-up, end = 1 adds its duration to map 0's statistics.
 __global__ void k_setup_stamp(const PcgArgs* pa, int end) {
@@ -37,11 +53,12 @@ __global__ void k_setup_stamp(const PcgArgs* pa, int end) {
 }
 
 // one warp per tile (grid-stride), the single map of the plan
-#define FCG_TILE_LOOP(a)                                               \
+#define FCG_TILE_LOOP(f)                                               \
   const int lane = threadIdx.x & 31;                                   \
   const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);  \
   const int NW = gridDim.x * (blockDim.x >> 5);                        \
-  const MapDesc& M = a.maps[0];                                        \
+  const PcgArgs& a = f.a;                                              \
+  const MapDesc& M = f.M;                                              \
   MapState* S = a.st;                                                  \
   for (int t = gw; t < a.ntiles; t += NW)
 
@@ -61,32 +78,111 @@ __device__ __forceinline__ void put_rbf(const PcgArgs& a, const MapDesc& M, int 
         make_float2((float)r.x, j + 1 < M.W ? (float)r.y : 0.f);
 }
 
-// The WHILE loop's own guard (one thread), run after the start phase and at the
-// head of every body execution: a map that has stopped -- or was never active in
-// this outer pass, so no finisher will run -- clears the condition, and so does
-// a loop that has run past l_max (reported as a time-out).  The rest of that body
-// execution then finds the map stopped and returns at once.
-__global__ void k_f_guard(const PcgArgs* pa, int count) {
-  const PcgArgs a = *pa;
-  MapState* S = a.st;
-  const MapDesc& M = a.maps[0];
-  const long long lmax = a.lmax > 0 ? a.lmax : 2LL * M.H * M.W;
-  const long long loops = count ? ++S->loops : S->loops;
-  if (*(volatile int*)&S->done) {
-    cudaGraphSetConditional(a.cond, 0);
-  } else if (loops > lmax + 2) {
-    S->status = -4;
-    S->done = 1;
-    atomicSub(a.n_active, 1);
-    __threadfence();
-    cudaGraphSetConditional(a.cond, 0);
+// The solve's scalars.  The kernels that make a dot product leave its partials, one per tile
+// or per unit of the multigrid cycle's last kernel, and whoever needs the scalar next adds
+// them, in tile_arrive's order: every block of phase B adds d^T q for its alpha, and the last
+// kernel of the start and of every body, one block, adds r^T s, r^T r and r_{k+1}^T s_k (or
+// b^T b) and runs the stop tests.  Counting the tiles in and electing a last warp to add them
+// was the serial end of those kernels, in which every other SM idled (ncu at 2048x2048: the
+// SMs active for 46,000 of k_x_a's 62,800 cycles and of the last cycle kernel's 67,000).
+// Mixed multigrid, us a call, before / after, with the set-up kernels' cheaper FP64 work:
+// 256x256 1825 / 1626, 2048x2048 11062 / 10376; twelve uneven maps 18677 / 17410.
+// The mixed form, whose iterates do not depend on how the sums are grouped (its scalars are
+// rounded to FP32), makes one partial per block instead of per tile: one SM adds 512 FP64
+// values in 0.4 us, the 4096 tiles of a 4096x4096 map in 3.
+constexpr int kSumThreads = 128;  // threads that add one array of partials
+
+// The mixed form's partials per block (the persistent solvers' slots, idle here): q = 0 d^T q,
+// 1 r^T r, 2 r_{k+1}^T s_k or b^T b.
+__device__ __forceinline__ double* block_part(const PcgArgs& a, int q) { return a.flow + (size_t)q * a.nflow; }
+
+// Sums of N lane values over the block into out[q][blockIdx.x]; all threads call, once.
+template <int N>
+__device__ __forceinline__ void put_block_parts(const double (&v)[N], double* const (&out)[N]) {
+  __shared__ double sh[N][kWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    const double s = warp_sum(v[q]);
+    if (lane == 0) sh[q][warp] = s;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    if (warp != q) continue;  // a warp per sum
+    double s = lane < kWarps ? sh[q][lane] : 0.0;
+#pragma unroll
+    for (int o = kWarps / 2; o > 0; o >>= 1) s += __shfl_down_sync(kFull, s, o);
+    if (lane == 0) __stcg(out[q] + blockIdx.x, s);
   }
 }
 
+// alpha = delta / d^T q from n partials in every thread of the block (all of them call);
+// block 0 records it.
+__device__ __forceinline__ double block_alpha(const PcgArgs& a, const MapDesc& M, MapState* S, const double* P, int n) {
+  __shared__ double part[kArriveGroups];
+  __shared__ double s_alpha;
+  const ScalarIn in = threadIdx.x == 0 ? load_scalars(S) : ScalarIn{};
+  if (threadIdx.x < kSumThreads) group_sums(P, n, threadIdx.x, part);
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const double dq = warp_sum(part[threadIdx.x]);
+    if (threadIdx.x == 0) {
+      const bool down = !(dq > 0.0) || !isfinite(dq);
+      s_alpha = down ? 0.0 : in.delta / dq;
+      if (blockIdx.x == 0) finish_scalars(a, M, S, in, kPhA, dq, 0.0, 0.0);
+    }
+  }
+  __syncthreads();
+  return s_alpha;
+}
+
+// The end of the start phase (ph = kPhResInit) or of a body (kPhFcg): n[q] partials of r^T s
+// (q = 0), r^T r (1) and the third sum (2), in P0, P1, P2 or, where blocks has bit q, in the
+// mixed form's per-block arrays.  Then the WHILE
+// loop's guard: a map that has stopped -- or was never active in this outer pass -- clears the
+// condition, and so does a loop that has run past l_max (reported as a time-out).
+__global__ void __launch_bounds__(3 * kSumThreads) k_f_finish(const __grid_constant__ FcgArgs f, int ph, int n0, int n1, int n2,
+                                                              int blocks) {
+  __shared__ double part[3][kArriveGroups];
+  __shared__ double sum[3];
+  MapState* S = f.a.st;
+  const MapDesc& M = f.M;
+  int done = *(volatile int*)&S->done;
+  const PcgArgs a = call_args(f);
+  const ScalarIn in = threadIdx.x == 0 ? load_scalars(S) : ScalarIn{};
+  if (!done) {
+    const int q = threadIdx.x / kSumThreads, r = threadIdx.x % kSumThreads;
+    const double* P = (blocks >> q & 1) ? block_part(a, q) : q == 0 ? a.P0 : q == 1 ? a.P1 : a.P2;
+    group_sums(P, q == 0 ? n0 : q == 1 ? n1 : n2, r, part[q]);
+    __syncthreads();
+    if (r < 32) {
+      const double v = warp_sum(part[q][r]);
+      if (r == 0) sum[q] = v;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x != 0) return;
+  if (!done && finish_scalars(a, M, S, in, ph, sum[0], sum[1], sum[2])) {
+    done = 1;
+    S->done = 1;
+    atomicSub(a.n_active, 1);
+  }
+  const long long lmax = a.lmax > 0 ? a.lmax : 2LL * M.H * M.W;
+  const long long loops = in.loops + (ph == kPhFcg ? 1 : 0);
+  S->loops = loops;
+  if (!done && loops > lmax + 2) {
+    S->status = -4;
+    S->done = 1;
+    atomicSub(a.n_active, 1);
+    done = 1;
+  }
+  if (done && a.cond) cudaGraphSetConditional(a.cond, 0);
+}
+
 // r = b - A phi (start, or refresh iterations only); on refresh iterations also r^T s_k.
-__global__ void __launch_bounds__(kThreads, 2) k_f_res(const PcgArgs* pa, int refresh_only) {
-  const PcgArgs a = *pa;
-  FCG_TILE_LOOP(a) {
+__global__ void __launch_bounds__(kThreads, 2) k_f_res(const __grid_constant__ FcgArgs f, int refresh_only) {
+  FCG_TILE_LOOP(f) {
     if (*(volatile int*)&S->done) return;
     const long long it = *(volatile long long*)&S->iter;
     if (refresh_only && (it % M.refresh) != 0) return;
@@ -114,12 +210,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_f_res(const PcgArgs* pa, int re
   }
 }
 
-// d = s + beta d_old (d = s at l = 0), q = A d, d^T q -> alpha.
-__global__ void __launch_bounds__(kThreads) k_f_a(const PcgArgs* pa) {
-  const PcgArgs a = *pa;
-  FCG_TILE_LOOP(a) {
+// d = s + beta d_old (d = s at l = 0), q = A d, d^T q per tile.
+__global__ void __launch_bounds__(kThreads) k_f_a(const __grid_constant__ FcgArgs f) {
+  FCG_TILE_LOOP(f) {
     if (*(volatile int*)&S->done) return;
-    a_tile<kJacobi>(a, M, S, t, lane);
+    const double dq = warp_sum(a_tile_dq<kJacobi>(a, M, t, *(volatile long long*)&S->iter,
+                                                  *(volatile double*)&S->beta, lane));
+    if (lane == 0) __stcg(a.P0 + t, dq);
   }
 }
 
@@ -137,110 +234,93 @@ __device__ __forceinline__ void cpa16f(void* sdst, const void* gsrc) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gsrc) : "memory");
 }
 
-// phi += alpha d; r -= alpha q and r^T s_k (not on refresh iterations).
-__global__ void __launch_bounds__(kThreads) k_f_b(const PcgArgs* pa) {
+// alpha; phi += alpha d; r -= alpha q and r^T s_k (not on refresh iterations).  One tile per warp.
+__global__ void __launch_bounds__(kThreads) k_f_b(const __grid_constant__ FcgArgs f) {
   extern __shared__ __align__(16) unsigned char fb_dsm[];
-  const PcgArgs a = *pa;
-  FCG_TILE_LOOP(a) {
-    if (*(volatile int*)&S->done) return;
-    const long long it = *(volatile long long*)&S->iter;
-    const bool refresh = (it % M.refresh) == 0;
-    const TileGeo g = tile_geo(M, t, a.R);
-    const size_t P = M.pitch;
-    const double* __restrict__ d = (it & 1) ? M.f.d0 : M.f.d1;
-    double* __restrict__ phi = M.f.phi;
-    double* __restrict__ rp = M.f.r;
-    const double* __restrict__ qp = M.f.q;
-    const double* __restrict__ sp = M.f.s;
-    const double alpha = *(volatile double*)&S->alpha;
-    const int j = g.j0 + 2 * lane;
-    double rsp = 0.0;
-    if (!refresh) {
-      // the rows stream through the warp's ring in shared memory, kLeadF rows ahead of
-      // the arithmetic (that of the loop below)
-      SlotF* ring = reinterpret_cast<SlotF*>(fb_dsm) + (threadIdx.x >> 5) * kRingF;
-      auto issue = [&](SlotF& sl, int i) {
-        const size_t off = (size_t)i * P + j;
-        cpa16f(&sl.d[lane], d + off);
-        cpa16f(&sl.ph[lane], phi + off);
-        cpa16f(&sl.q[lane], qp + off);
-        cpa16f(&sl.s[lane], sp + off);
-        cpa16f(&sl.r[lane], rp + off);
-      };
+  const PcgArgs& a = f.a;
+  const int lane = threadIdx.x & 31;
+  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const MapDesc& M = f.M;
+  MapState* S = a.st;
+  if (*(volatile int*)&S->done) return;
+  const long long it = *(volatile long long*)&S->iter;
+  const bool refresh = (it % M.refresh) == 0;
+  const bool have = t < a.ntiles;
+  const TileGeo g = tile_geo(M, have ? t : 0, a.R);
+  const size_t P = M.pitch;
+  const double* __restrict__ d = (it & 1) ? M.f.d0 : M.f.d1;
+  double* __restrict__ phi = M.f.phi;
+  double* __restrict__ rp = M.f.r;
+  const double* __restrict__ qp = M.f.q;
+  const double* __restrict__ sp = M.f.s;
+  const int j = g.j0 + 2 * lane;
+  // the rows stream through the warp's ring in shared memory, kLeadF rows ahead of the
+  // arithmetic; the first ones are under way while the block adds up alpha
+  SlotF* ring = reinterpret_cast<SlotF*>(fb_dsm) + (threadIdx.x >> 5) * kRingF;
+  auto issue = [&](SlotF& sl, int i) {
+    const size_t off = (size_t)i * P + j;
+    cpa16f(&sl.d[lane], d + off);
+    cpa16f(&sl.ph[lane], phi + off);
+    cpa16f(&sl.q[lane], qp + off);
+    cpa16f(&sl.s[lane], sp + off);
+    cpa16f(&sl.r[lane], rp + off);
+  };
 #pragma unroll
-      for (int k = 0; k < kLeadF; ++k) {
-        if (g.i0 + k < g.i1) issue(ring[k], g.i0 + k);
-        cpa_commit();
-      }
-      for (int i = g.i0; i < g.i1; ++i) {
-        cpa_wait<kLeadF - 1>();
-        const SlotF& sl = ring[(i - g.i0) % kRingF];
-        const double2 dv = sl.d[lane], qv = sl.q[lane], sv = sl.s[lane];
-        double2 ph = sl.ph[lane], r = sl.r[lane];
-        if (i + kLeadF < g.i1) issue(ring[(i + kLeadF - g.i0) % kRingF], i + kLeadF);
-        cpa_commit();
-        const size_t off = (size_t)i * P + j;
-        ph.x = fma(alpha, dv.x, ph.x);
-        ph.y = fma(alpha, dv.y, ph.y);
-        st2(phi, off, ph);
-        r.x = fma(-alpha, qv.x, r.x);
-        r.y = fma(-alpha, qv.y, r.y);
-        st2(rp, off, r);
-        put_rbf(a, M, i, j, r);
-        rsp = fma(r.x, sv.x, rsp);
-        rsp = fma(r.y, sv.y, rsp);
-      }
-      cpa_wait_all();  // the warp's next tile refills the same slots
-      rsp = warp_sum(rsp);
-      if (lane == 0) __stcg(a.P2 + t, rsp);
-      continue;
-    }
-    // refresh iterations (phi only): rows in groups of four, all loads of a group first
+  for (int k = 0; k < kLeadF; ++k) {
+    if (have && !refresh && g.i0 + k < g.i1) issue(ring[k], g.i0 + k);
+    cpa_commit();
+  }
+  const double alpha = block_alpha(a, M, S, a.P0 + M.tile_base, M.ntiles);
+  if (!have) return;
+  if (refresh) {
+    // phi only: rows in groups of four, all loads of a group first
     for (int i = g.i0; i < g.i1; i += 4) {
-      double2 dv[4], ph[4], qv[4], sv[4], rv[4];
+      double2 dv[4], ph[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         if (i + k < g.i1) {
           const size_t off = (size_t)(i + k) * P + j;
           dv[k] = ld2(d, off);
           ph[k] = ld2(phi, off);
-          if (!refresh) {
-            qv[k] = ld2(qp, off);
-            sv[k] = ld2(sp, off);
-            rv[k] = ld2(rp, off);
-          }
         }
       }
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         if (i + k < g.i1) {
-          const size_t off = (size_t)(i + k) * P + j;
           ph[k].x = fma(alpha, dv[k].x, ph[k].x);
           ph[k].y = fma(alpha, dv[k].y, ph[k].y);
-          st2(phi, off, ph[k]);
-          if (!refresh) {
-            double2 r = rv[k];
-            r.x = fma(-alpha, qv[k].x, r.x);
-            r.y = fma(-alpha, qv[k].y, r.y);
-            st2(rp, off, r);
-            put_rbf(a, M, i + k, j, r);
-            rsp = fma(r.x, sv[k].x, rsp);
-            rsp = fma(r.y, sv[k].y, rsp);
-          }
+          st2(phi, (size_t)(i + k) * P + j, ph[k]);
         }
       }
     }
-    if (!refresh) {
-      rsp = warp_sum(rsp);
-      if (lane == 0) __stcg(a.P2 + t, rsp);
-    }
+    return;
   }
+  double rsp = 0.0;
+  for (int i = g.i0; i < g.i1; ++i) {
+    cpa_wait<kLeadF - 1>();
+    const SlotF& sl = ring[(i - g.i0) % kRingF];
+    const double2 dv = sl.d[lane], qv = sl.q[lane], sv = sl.s[lane];
+    double2 ph = sl.ph[lane], r = sl.r[lane];
+    if (i + kLeadF < g.i1) issue(ring[(i + kLeadF - g.i0) % kRingF], i + kLeadF);
+    cpa_commit();
+    const size_t off = (size_t)i * P + j;
+    ph.x = fma(alpha, dv.x, ph.x);
+    ph.y = fma(alpha, dv.y, ph.y);
+    st2(phi, off, ph);
+    r.x = fma(-alpha, qv.x, r.x);
+    r.y = fma(-alpha, qv.y, r.y);
+    st2(rp, off, r);
+    put_rbf(a, M, i, j, r);
+    rsp = fma(r.x, sv.x, rsp);
+    rsp = fma(r.y, sv.y, rsp);
+  }
+  rsp = warp_sum(rsp);
+  if (lane == 0) __stcg(a.P2 + t, rsp);
 }
 
-// r^T s, r^T r (and b^T b at the start) -> delta, beta, stop test.
-__global__ void __launch_bounds__(kThreads, 2) k_f_dots(const PcgArgs* pa, int init) {
-  const PcgArgs a = *pa;
-  FCG_TILE_LOOP(a) {
+// r^T s, r^T r (and b^T b at the start) per tile.
+__global__ void __launch_bounds__(kThreads, 2) k_f_dots(const __grid_constant__ FcgArgs f, int init) {
+  FCG_TILE_LOOP(f) {
     if (*(volatile int*)&S->done) return;
     const TileGeo g = tile_geo(M, t, a.R);
     const size_t P = M.pitch;
@@ -283,7 +363,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_f_dots(const PcgArgs* pa, int i
         }
       }
     }
-    tile_arrive(a, M, S, t, init ? kPhResInit : kPhFcg, rs, rr, bb, lane);
+    rs = warp_sum(rs);
+    rr = warp_sum(rr);
+    if (init) bb = warp_sum(bb);
+    if (lane == 0) {
+      __stcg(a.P0 + t, rs);
+      __stcg(a.P1 + t, rr);
+      if (init) __stcg(a.P2 + t, bb);  // else r_{k+1}^T s_k from phase B
+    }
   }
 }
 
@@ -318,7 +405,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_f_dots(const PcgArgs* pa, int i
 // confirmation that missed it.
 struct XState {
   long long it;
-  double alpha;
   int done, confirm, refresh;
 };
 __device__ __forceinline__ XState x_state(const MapDesc& M, MapState* S) {
@@ -329,20 +415,24 @@ __device__ __forceinline__ XState x_state(const MapDesc& M, MapState* S) {
   const int fr = v->force_refresh;
   x.confirm = v->confirm;
   const int rn = v->refresh_next;
-  x.alpha = v->alpha;
   x.refresh = ((x.it > 0 && (x.it % M.refresh) == 0) ? 1 : 0) | fr | x.confirm | rn;
   return x;
 }
 
-__global__ void __launch_bounds__(kThreads, 2) k_x_a(const PcgArgs* pa) {
+// One tile per warp.
+__global__ void __launch_bounds__(kThreads, 2) k_x_a(const __grid_constant__ FcgArgs f) {
   __shared__ Slot32 ring[kWarps][kRing32];  // the stencil's row rings
-  const PcgArgs a = *pa;
-  FCG_TILE_LOOP(a) {
-    const volatile MapState* v = S;
-    const int done = v->done, confirm = v->confirm;
-    if (done | confirm) return;  // a confirmation body takes no step
-    a32_tile<kJacobi>(a, M, S, t, lane, ring[threadIdx.x >> 5]);
-  }
+  const PcgArgs& a = f.a;
+  const int lane = threadIdx.x & 31;
+  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const volatile MapState* v = a.st;
+  const int done = v->done, confirm = v->confirm;
+  const long long it = v->iter;
+  const double beta = v->beta;
+  if (done | confirm) return;  // a confirmation body takes no step
+  double dq = 0.0;
+  if (t < a.ntiles) dq = a32_tile_dq<kJacobi>(a, f.M, t, it, beta, lane, ring[threadIdx.x >> 5]);
+  put_block_parts<1>({dq}, {block_part(a, 0)});
 }
 
 // Phase B's row ring: kRingB slots per warp of the five FP32 rows it reads (dynamic
@@ -354,117 +444,119 @@ struct SlotB {
 };
 constexpr size_t kRingBSmem = (size_t)kWarps * kRingB * sizeof(SlotB);  // 71,680 bytes
 
-__global__ void __launch_bounds__(kThreads, 2) k_x_b(const PcgArgs* pa) {
+// alpha, then the phase's updates.  One tile per warp.
+__global__ void __launch_bounds__(kThreads, 2) k_x_b(const __grid_constant__ FcgArgs f) {
   extern __shared__ __align__(16) unsigned char xb_dsm[];
-  const PcgArgs a = *pa;
-  FCG_TILE_LOOP(a) {
-    const XState xs = x_state(M, S);
-    if (xs.done) return;
-    const bool refresh = xs.refresh;
-    const long long it = xs.it;
-    const TileGeo g = tile_geo(M, t, a.R);
-    const size_t P = M.pitch;
-    const float* __restrict__ d = (it & 1) ? M.h.d0 : M.h.d1;
-    // a confirmation body only folds the correction into phi (no step: alpha = 0)
-    const float alpha = xs.confirm ? 0.f : (float)xs.alpha;
-    const int j = g.j0 + 2 * lane;
-    DF rsp, rrp;
-    if (refresh) {
-      // phi += x + alpha d, x = 0: rows in groups of four, all loads of a group first
-      for (int i = g.i0; i < g.i1; i += 4) {
-        float2 dv[4], xv[4];
-        double2 pv[4];
+  const PcgArgs& a = f.a;
+  const int lane = threadIdx.x & 31;
+  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const MapDesc& M = f.M;
+  MapState* S = a.st;
+  const XState xs = x_state(M, S);
+  if (xs.done) return;
+  const bool have = t < a.ntiles;
+  const bool refresh = xs.refresh;
+  const TileGeo g = tile_geo(M, have ? t : 0, a.R);
+  const size_t P = M.pitch;
+  const float* __restrict__ d = (xs.it & 1) ? M.h.d0 : M.h.d1;
+  const int j = g.j0 + 2 * lane;
+  // the five rows of each pixel row stream through the warp's ring in shared memory, kLeadB
+  // rows ahead of the arithmetic (the loads in flight cost no registers, and each lane reads
+  // back only what it copied); the first ones are under way while the block adds up alpha
+  SlotB* ring = reinterpret_cast<SlotB*>(xb_dsm) + (threadIdx.x >> 5) * kRingB;
+  auto issue = [&](SlotB& sl, int i) {
+    const size_t off = (size_t)i * P + j;
+    cpa8(&sl.d[lane], d + off, 8);
+    cpa8(&sl.x[lane], M.h.x + off, 8);
+    cpa8(&sl.q[lane], M.h.q + off, 8);
+    cpa8(&sl.r[lane], M.h.r + off, 8);
+    cpa8(&sl.s[lane], M.h.s + off, 8);
+  };
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (i + k < g.i1) {
-            const size_t off = (size_t)(i + k) * P + j;
-            dv[k] = ldf2(d, off);
-            xv[k] = ldf2(M.h.x, off);
-            pv[k] = ld2(M.f.phi, off);
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (i + k < g.i1) {
-            const size_t off = (size_t)(i + k) * P + j;
-            float2 x = xv[k];
-            x.x = __fmaf_rn(alpha, dv[k].x, x.x);
-            x.y = __fmaf_rn(alpha, dv[k].y, x.y);
-            double2 ph = pv[k];
-            ph.x += (double)x.x;
-            ph.y += (double)x.y;
-            st2(M.f.phi, off, ph);
-            stf2(M.h.x, off, make_float2(0.f, 0.f));
-          }
-        }
-      }
-    } else {
-      // x += alpha d, r -= alpha q and the partials r^T s, r^T r: the five rows of
-      // each pixel row stream through the warp's ring in shared memory, kLeadB rows
-      // ahead of the arithmetic (the loads in flight cost no registers, and each lane
-      // reads back only what it copied)
-      SlotB* ring = reinterpret_cast<SlotB*>(xb_dsm) + (threadIdx.x >> 5) * kRingB;
-      auto issue = [&](SlotB& sl, int i) {
-        const size_t off = (size_t)i * P + j;
-        cpa8(&sl.d[lane], d + off, 8);
-        cpa8(&sl.x[lane], M.h.x + off, 8);
-        cpa8(&sl.q[lane], M.h.q + off, 8);
-        cpa8(&sl.r[lane], M.h.r + off, 8);
-        cpa8(&sl.s[lane], M.h.s + off, 8);
-      };
-#pragma unroll
-      for (int k = 0; k < kLeadB; ++k) {
-        if (g.i0 + k < g.i1) issue(ring[k], g.i0 + k);
-        cpa_commit();
-      }
-      for (int i = g.i0; i < g.i1; ++i) {
-        cpa_wait<kLeadB - 1>();  // row i has landed
-        const SlotB& sl = ring[(i - g.i0) % kRingB];
-        const float2 dv = sl.d[lane], qv = sl.q[lane], sv = sl.s[lane];
-        float2 x = sl.x[lane], r = sl.r[lane];
-        // the slot of row i - 1 is free: refill it with row i + kLeadB
-        if (i + kLeadB < g.i1) issue(ring[(i + kLeadB - g.i0) % kRingB], i + kLeadB);
-        cpa_commit();
-        const size_t off = (size_t)i * P + j;
-        x.x = __fmaf_rn(alpha, dv.x, x.x);
-        x.y = __fmaf_rn(alpha, dv.y, x.y);
-        stf2(M.h.x, off, x);
-        r.x = __fmaf_rn(-alpha, qv.x, r.x);
-        r.y = __fmaf_rn(-alpha, qv.y, r.y);
-        stf2(M.h.r, off, r);
-        rsp.add_prod(r.x, sv.x);
-        rsp.add_prod(r.y, sv.y);
-        rrp.add_prod(r.x, r.x);
-        rrp.add_prod(r.y, r.y);
-      }
-      cpa_wait_all();  // the warp's next tile refills the same slots
-    }
-    if (!refresh) {
-      // r_{k+1}^T s_k and r_{k+1}^T r_{k+1} per tile for the dot phase
-      const double v = warp_sum(rsp.value()), w = warp_sum(rrp.value());
-      if (lane == 0) {
-        __stcg(a.P2 + t, v);
-        __stcg(a.P1 + t, w);
-      }
-    }
+  for (int k = 0; k < kLeadB; ++k) {
+    if (have && !refresh && g.i0 + k < g.i1) issue(ring[k], g.i0 + k);
+    cpa_commit();
   }
+  // a confirmation body only folds the correction into phi (no phase A, no step: alpha = 0)
+  const float alpha = xs.confirm ? 0.f : (float)block_alpha(a, M, S, block_part(a, 0), gridDim.x);
+  if (refresh) {
+    if (!have) return;
+    // phi += x + alpha d, x = 0: rows in groups of four, all loads of a group first
+    for (int i = g.i0; i < g.i1; i += 4) {
+      float2 dv[4], xv[4];
+      double2 pv[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (i + k < g.i1) {
+          const size_t off = (size_t)(i + k) * P + j;
+          dv[k] = ldf2(d, off);
+          xv[k] = ldf2(M.h.x, off);
+          pv[k] = ld2(M.f.phi, off);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (i + k < g.i1) {
+          const size_t off = (size_t)(i + k) * P + j;
+          float2 x = xv[k];
+          x.x = __fmaf_rn(alpha, dv[k].x, x.x);
+          x.y = __fmaf_rn(alpha, dv[k].y, x.y);
+          double2 ph = pv[k];
+          ph.x += (double)x.x;
+          ph.y += (double)x.y;
+          st2(M.f.phi, off, ph);
+          stf2(M.h.x, off, make_float2(0.f, 0.f));
+        }
+      }
+    }
+    return;
+  }
+  // x += alpha d, r -= alpha q and the partials r_{k+1}^T s_k, r^T r for the dot phase
+  DF rsp, rrp;
+  const int i1 = have ? g.i1 : g.i0;
+  for (int i = g.i0; i < i1; ++i) {
+    cpa_wait<kLeadB - 1>();  // row i has landed
+    const SlotB& sl = ring[(i - g.i0) % kRingB];
+    const float2 dv = sl.d[lane], qv = sl.q[lane], sv = sl.s[lane];
+    float2 x = sl.x[lane], r = sl.r[lane];
+    // the slot of row i - 1 is free: refill it with row i + kLeadB
+    if (i + kLeadB < g.i1) issue(ring[(i + kLeadB - g.i0) % kRingB], i + kLeadB);
+    cpa_commit();
+    const size_t off = (size_t)i * P + j;
+    x.x = __fmaf_rn(alpha, dv.x, x.x);
+    x.y = __fmaf_rn(alpha, dv.y, x.y);
+    stf2(M.h.x, off, x);
+    r.x = __fmaf_rn(-alpha, qv.x, r.x);
+    r.y = __fmaf_rn(-alpha, qv.y, r.y);
+    stf2(M.h.r, off, r);
+    rsp.add_prod(r.x, sv.x);
+    rsp.add_prod(r.y, sv.y);
+    rrp.add_prod(r.x, r.x);
+    rrp.add_prod(r.y, r.y);
+  }
+  put_block_parts<2>({rsp.value(), rrp.value()}, {block_part(a, 2), block_part(a, 1)});
 }
 
 // r = b - A phi in FP64, rounded to FP32, and its r^T r per tile (x = 0 with it at the
 // start, and the b^T b partials for the start's dot phase); on refresh iterations also
 // r_{k+1}^T s_k.
-__global__ void __launch_bounds__(kThreads, 2) k_x_res(const PcgArgs* pa, int init) {
-  const PcgArgs a = *pa;
-  FCG_TILE_LOOP(a) {
-    const XState xs = x_state(M, S);
-    if (xs.done) return;
-    if (!init && !xs.refresh) return;
-    // a confirmation body under the relative-residual stop decides here whether the solve ends
-    const bool confirm = !init && a.stop_mode == ULP_STOP_RELRES && xs.confirm;
+// One tile per warp.
+__global__ void __launch_bounds__(kThreads, 2) k_x_res(const __grid_constant__ FcgArgs f, int init) {
+  const PcgArgs& a = f.a;
+  const int lane = threadIdx.x & 31;
+  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const MapDesc& M = f.M;
+  MapState* S = a.st;
+  const XState xs = x_state(M, S);
+  if (xs.done) return;
+  if (!init && !xs.refresh) return;
+  // a confirmation body under the relative-residual stop decides here whether the solve ends
+  const bool confirm = !init && a.stop_mode == ULP_STOP_RELRES && xs.confirm;
+  DF rsp, rrp;
+  double bb = 0.0;
+  if (t < a.ntiles) {
     const TileGeo g = tile_geo(M, t, a.R);
     XPlane x{M.f.phi, (size_t)M.pitch};
-    DF rsp, rrp;
-    double bb = 0.0;
     auto epi = [&](size_t off, double2, double2 ax) {
       const double2 bv = ld2(M.f.b, off);
       const float2 r = make_float2((float)(bv.x - ax.x), (float)(bv.y - ax.y));
@@ -482,26 +574,16 @@ __global__ void __launch_bounds__(kThreads, 2) k_x_res(const PcgArgs* pa, int in
       }
     };
     stencil_tile(M, g.i0, g.i1, g.j0, lane, M.f.U, M.f.V, M.f.D, x, epi);
-    const double v = warp_sum(init ? bb : rsp.value());
-    if (confirm) {
-      // r_{k+1}^T s_k for the dot phase, should the body go on; r^T r through the arrival
-      if (lane == 0) __stcg(a.P2 + t, v);
-      tile_arrive(a, M, S, t, kPhConfirm, 0.0, rrp.value(), 0.0, lane);
-      continue;
-    }
-    const double w = warp_sum(rrp.value());
-    if (lane == 0) {
-      __stcg(a.P2 + t, v);
-      __stcg(a.P1 + t, w);
-    }
   }
+  // r_{k+1}^T s_k (b^T b at the start) and r^T r for the dot phase
+  put_block_parts<2>({init ? bb : rsp.value(), rrp.value()}, {block_part(a, 2), block_part(a, 1)});
+  if (confirm && t < a.ntiles) tile_arrive(call_args(f), M, S, t, kPhConfirm, 0.0, rrp.value(), 0.0, lane);
 }
 
 // r^T s, r^T r (double-float) and, at the start of the solve, b^T b (FP64) -> delta, beta,
 // stop test (used where the multigrid cycle cannot carry the dot phase)
-__global__ void __launch_bounds__(kThreads, 2) k_x_dots(const PcgArgs* pa, int init) {
-  const PcgArgs a = *pa;
-  FCG_TILE_LOOP(a) {
+__global__ void __launch_bounds__(kThreads, 2) k_x_dots(const __grid_constant__ FcgArgs f, int init) {
+  FCG_TILE_LOOP(f) {
     if (*(volatile int*)&S->done) return;
     const TileGeo g = tile_geo(M, t, a.R);
     const size_t P = M.pitch;
@@ -521,18 +603,24 @@ __global__ void __launch_bounds__(kThreads, 2) k_x_dots(const PcgArgs* pa, int i
         bb = fma(bv.y, bv.y, bb);
       }
     }
-    tile_arrive(a, M, S, t, init ? kPhResInit : kPhFcg, rs.value(), rr.value(), bb, lane);
+    const double vs = warp_sum(rs.value()), vr = warp_sum(rr.value());
+    if (init) bb = warp_sum(bb);
+    if (lane == 0) {
+      __stcg(a.P0 + t, vs);
+      __stcg(a.P1 + t, vr);
+      if (init) __stcg(a.P2 + t, bb);
+    }
   }
 }
 
 // end of the solve: phi += x; nothing to do after a stop on a refresh iteration (x = 0 then),
 // only after l_max or a breakdown
-__global__ void __launch_bounds__(kThreads) k_x_fold(const PcgArgs* pa) {
-  const PcgArgs a = *pa;
+__global__ void __launch_bounds__(kThreads) k_x_fold(const __grid_constant__ FcgArgs f) {
+  const PcgArgs& a = f.a;
   const int lane = threadIdx.x & 31;
   const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int NW = gridDim.x * (blockDim.x >> 5);
-  const MapDesc& M = a.maps[0];
+  const MapDesc& M = f.M;
   if (!a.st->outer_active || *(volatile int*)&a.st->x_clean) return;
   for (int t = gw; t < a.ntiles; t += NW) {
     const TileGeo g = tile_geo(M, t, a.R);
@@ -552,9 +640,8 @@ __global__ void __launch_bounds__(kThreads) k_x_fold(const PcgArgs* pa) {
 
 // Learned preconditioner's fallback: s = D^-1 r once the map's fallback flag is
 // set (the network kernels skip themselves from then on).
-__global__ void __launch_bounds__(kThreads) k_f_jacobi(const PcgArgs* pa) {
-  const PcgArgs a = *pa;
-  FCG_TILE_LOOP(a) {
+__global__ void __launch_bounds__(kThreads) k_f_jacobi(const __grid_constant__ FcgArgs f) {
+  FCG_TILE_LOOP(f) {
     if (*(volatile int*)&S->done || !*(volatile int*)&S->fallback) return;
     const TileGeo g = tile_geo(M, t, a.R);
     const size_t P = M.pitch;
@@ -579,74 +666,88 @@ static bool mixed_fcg(const Plan& pl, int kind) {
   return kind == ULP_PRECOND_MG && pl.opt.precision == ULP_PRECISION_MIXED;
 }
 
-// With fuse_dots the multigrid cycle's last kernel also runs the dot phase D (at the
-// start of a solve, init: its start form, with b^T b).
+// With fuse_dots the multigrid cycle's last kernel also leaves the dot phase's partials.
 // part (multigrid): as mg_apply's, so a replay can time the cycle's last kernel alone.
-static cudaError_t fcg_precond(Plan& pl, int kind, cudaStream_t st, bool fuse_dots = false, bool init = false,
+static cudaError_t fcg_precond(Plan& pl, int kind, const FcgArgs& f, cudaStream_t st, bool fuse_dots = false,
                                int part = 0) {
   const MapDesc& M = pl.hmaps[0];
   if (kind == ULP_PRECOND_DCT) return dct_apply(*pl.dct, M.f.r, M.pitch, M.f.mask, M.f.s, st, true);
   if (kind == ULP_PRECOND_MG)
-    return mg_apply(*pl.mg, M.f.mask, pl.dstate, st, true, fuse_dots ? pl.dargs : nullptr,
-                    mixed_fcg(pl, kind) ? M.h.s : nullptr, init, part);
+    return mg_apply(*pl.mg, M.f.mask, pl.dstate, st, true, fuse_dots ? &f.a : nullptr,
+                    mixed_fcg(pl, kind) ? M.h.s : nullptr, part);
   if (kind == ULP_PRECOND_RBSSOR || kind == ULP_PRECOND_RBILU) return rb_apply(pl, kind, pl.dstate, st);
   const cudaError_t e = unet_apply_plane(*pl.unet, M.f.r, M.f.U, M.f.V, M.f.mask, M.H, M.W, M.pitch, M.f.s,
                                          &pl.dstate[0].fallback, st);
   if (e != cudaSuccess) return e;
-  k_f_jacobi<<<tile_blocks(pl), kThreads, 0, st>>>(pl.dargs);
+  k_f_jacobi<<<tile_blocks(pl), kThreads, 0, st>>>(f);
   return cudaGetLastError();
 }
 
 // D rides on the multigrid cycle's last kernel where the plan allows it
 static bool fused_dots(const Plan& pl, int kind) { return kind == ULP_PRECOND_MG && mg_fuses_dots(*pl.mg); }
 
+// The scalars after the start (init) or a body's dot phase.
+static void fcg_finish(Plan& pl, int kind, const FcgArgs& f, bool fd, bool init, cudaStream_t st) {
+  const bool x = mixed_fcg(pl, kind);
+  const int nb = tile_blocks(pl), nt = pl.ntiles, nu = fd ? mg_dot_units(*pl.mg) : nt;
+  // r^T r comes from the dot phase's kernel, but in the fused mixed form from those that wrote
+  // r; the third sum from phase B, the residual, or k_f_dots / k_x_dots at the start
+  const bool b1 = x && fd, b2 = x && (fd || !init);
+  k_f_finish<<<1, 3 * kSumThreads, 0, st>>>(f, init ? kPhResInit : kPhFcg, nu, b1 ? nb : nu, b2 ? nb : nt,
+                                            (b1 ? 2 : 0) | (b2 ? 4 : 0));
+}
+
 // Start of a solve: r = b - A phi (and its BF16 copy), the mask bits, s = M^-1 r, delta_0.
-static cudaError_t fcg_start(Plan& pl, int kind, cudaStream_t st) {
+static cudaError_t fcg_start(Plan& pl, int kind, const FcgArgs& f, cudaStream_t st) {
   const MapDesc& M = pl.hmaps[0];
   const int nb = tile_blocks(pl);
   const bool stamp = pl.opt.profile != 0;
   if (mixed_fcg(pl, kind)) {
     const bool fd = fused_dots(pl, kind);
-    k_x_res<<<nb, kThreads, 0, st>>>(pl.dargs, 1);
+    k_x_res<<<nb, kThreads, 0, st>>>(f, 1);
     if (stamp) k_setup_stamp<<<1, 1, 0, st>>>(pl.dargs, 0);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = mg_setup(*pl.mg, pl.dstate, st, !pl.system_x);
     if (stamp) k_setup_stamp<<<1, 1, 0, st>>>(pl.dargs, 1);
-    if (e == cudaSuccess) e = fcg_precond(pl, kind, st, fd, true);
-    if (!fd) k_x_dots<<<nb, kThreads, 0, st>>>(pl.dargs, 1);
+    if (e == cudaSuccess) e = fcg_precond(pl, kind, f, st, fd);
+    if (!fd) k_x_dots<<<nb, kThreads, 0, st>>>(f, 1);
+    fcg_finish(pl, kind, f, fd, true, st);
     return e == cudaSuccess ? cudaGetLastError() : e;
   }
-  k_f_res<<<nb, kThreads, 0, st>>>(pl.dargs, 0);
+  k_f_res<<<nb, kThreads, 0, st>>>(f, 0);
   if (stamp) k_setup_stamp<<<1, 1, 0, st>>>(pl.dargs, 0);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && kind == ULP_PRECOND_DCT) e = dct_prepare_mask(*pl.dct, M.f.mask, M.pitch, st);
   if (e == cudaSuccess && kind == ULP_PRECOND_MG) e = mg_setup(*pl.mg, pl.dstate, st);
   if (e == cudaSuccess) e = rb_setup(pl, kind, pl.dstate, st);
   if (stamp) k_setup_stamp<<<1, 1, 0, st>>>(pl.dargs, 1);
-  if (e == cudaSuccess) e = fcg_precond(pl, kind, st);
-  k_f_dots<<<nb, kThreads, 0, st>>>(pl.dargs, 1);
+  if (e == cudaSuccess) e = fcg_precond(pl, kind, f, st);
+  k_f_dots<<<nb, kThreads, 0, st>>>(f, 1);
+  fcg_finish(pl, kind, f, false, true, st);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 // One iteration: A, B, R, s = M^-1 r, D.
-static cudaError_t fcg_iteration(Plan& pl, int kind, cudaStream_t st) {
+static cudaError_t fcg_iteration(Plan& pl, int kind, const FcgArgs& f, cudaStream_t st) {
   const int nb = tile_blocks(pl);
   const bool fd = fused_dots(pl, kind);
   if (mixed_fcg(pl, kind)) {
-    k_x_a<<<nb, kThreads, 0, st>>>(pl.dargs);
-    k_x_b<<<nb, kThreads, kRingBSmem, st>>>(pl.dargs);
-    k_x_res<<<nb, kThreads, 0, st>>>(pl.dargs, 0);
+    k_x_a<<<nb, kThreads, 0, st>>>(f);
+    k_x_b<<<nb, kThreads, kRingBSmem, st>>>(f);
+    k_x_res<<<nb, kThreads, 0, st>>>(f, 0);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = fcg_precond(pl, kind, st, fd);
-    if (!fd) k_x_dots<<<nb, kThreads, 0, st>>>(pl.dargs, 0);
+    if (e == cudaSuccess) e = fcg_precond(pl, kind, f, st, fd);
+    if (!fd) k_x_dots<<<nb, kThreads, 0, st>>>(f, 0);
+    fcg_finish(pl, kind, f, fd, false, st);
     return e == cudaSuccess ? cudaGetLastError() : e;
   }
-  k_f_a<<<nb, kThreads, 0, st>>>(pl.dargs);
-  k_f_b<<<nb, kThreads, kRingFSmem, st>>>(pl.dargs);
-  k_f_res<<<nb, kThreads, 0, st>>>(pl.dargs, 1);
+  k_f_a<<<nb, kThreads, 0, st>>>(f);
+  k_f_b<<<nb, kThreads, kRingFSmem, st>>>(f);
+  k_f_res<<<nb, kThreads, 0, st>>>(f, 1);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = fcg_precond(pl, kind, st, fd);
-  if (!fd) k_f_dots<<<nb, kThreads, 0, st>>>(pl.dargs, 0);
+  if (e == cudaSuccess) e = fcg_precond(pl, kind, f, st, fd);
+  if (!fd) k_f_dots<<<nb, kThreads, 0, st>>>(f, 0);
+  fcg_finish(pl, kind, f, fd, false, st);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
@@ -657,8 +758,8 @@ static cudaError_t fcg_attrs() {
   return cudaFuncSetAttribute(k_x_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingBSmem);
 }
 
-// Captures the solve graph: start, then WHILE { guard, iteration }.
-static cudaError_t fcg_build(Plan& pl, int kind) {
+// Captures the solve graph: start, then WHILE { iteration }.
+static cudaError_t fcg_build(Plan& pl, int kind, FcgArgs f) {
   cudaError_t e = fcg_attrs();
   if (e != cudaSuccess) return e;
   if (!pl.cap_stream) {
@@ -673,16 +774,14 @@ static cudaError_t fcg_build(Plan& pl, int kind) {
     cudaGraphDestroy(g);
     return e;
   }
-  pl.fcg_cond = h;
   cudaGraphNodeParams cp = {};
   if ((e = cudaStreamBeginCaptureToGraph(st, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal)) !=
       cudaSuccess) {
     cudaGraphDestroy(g);
     return e;
   }
-  e = fcg_start(pl, kind, st);
-  k_f_guard<<<1, 1, 0, st>>>(pl.dargs, 0);
-  if (e == cudaSuccess) e = cudaGetLastError();
+  f.a.cond = h;
+  e = fcg_start(pl, kind, f, st);
   cudaStreamCaptureStatus cs;
   const cudaGraphNode_t* deps = nullptr;
   size_t ndeps = 0;
@@ -697,7 +796,7 @@ static cudaError_t fcg_build(Plan& pl, int kind) {
   }
   if (e == cudaSuccess) e = cudaStreamUpdateCaptureDependencies(st, &cn, nullptr, 1, cudaStreamSetCaptureDependencies);
   if (e == cudaSuccess && mixed_fcg(pl, kind)) {
-    k_x_fold<<<tile_blocks(pl), kThreads, 0, st>>>(pl.dargs);
+    k_x_fold<<<tile_blocks(pl), kThreads, 0, st>>>(f);
     e = cudaGetLastError();
   }
   cudaGraph_t gout = nullptr;
@@ -710,8 +809,7 @@ static cudaError_t fcg_build(Plan& pl, int kind) {
   cudaGraph_t body = cp.conditional.phGraph_out[0];
   if ((e = cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal)) ==
       cudaSuccess) {
-    k_f_guard<<<1, 1, 0, st>>>(pl.dargs, 1);
-    e = fcg_iteration(pl, kind, st);
+    e = fcg_iteration(pl, kind, f, st);
     cudaGraph_t bout = nullptr;
     const cudaError_t e3 = cudaStreamEndCapture(st, &bout);
     if (e == cudaSuccess) e = e3;
@@ -736,62 +834,19 @@ static cudaError_t fcg_build(Plan& pl, int kind) {
 // Host-driven form of the same solve (options.profile = 2): every kernel is a
 // host launch, so a profiler sees each one; the host reads the stop flag after
 // every iteration.  For measurement only.
-static cudaError_t fcg_eager_mixed(Plan& pl, int kind, cudaStream_t st) {
+static cudaError_t fcg_eager_mixed(Plan& pl, int kind, const FcgArgs& f, cudaStream_t st) {
   const int nb = tile_blocks(pl);
   const bool fd = fused_dots(pl, kind);
   cudaError_t e = fcg_attrs();
   if (e != cudaSuccess) return e;
   phase_mark(pl, st, -1);
-  k_x_res<<<nb, kThreads, 0, st>>>(pl.dargs, 1);
+  k_x_res<<<nb, kThreads, 0, st>>>(f, 1);
   phase_mark(pl, st, 2);
   if ((e = mg_setup(*pl.mg, pl.dstate, st, !pl.system_x)) != cudaSuccess) return e;
-  if ((e = fcg_precond(pl, kind, st, fd, true)) != cudaSuccess) return e;
+  if ((e = fcg_precond(pl, kind, f, st, fd)) != cudaSuccess) return e;
   phase_mark(pl, st, 3);
-  if (!fd) {
-    k_x_dots<<<nb, kThreads, 0, st>>>(pl.dargs, 1);
-    phase_mark(pl, st, 4);
-  }
-  for (long long l = 0;; ++l) {
-    int done = 0;
-    if ((e = cudaMemcpyAsync(&done, &pl.dstate->done, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-    if (done || l > (1LL << 24)) break;
-    phase_mark(pl, st, -1);
-    k_x_a<<<nb, kThreads, 0, st>>>(pl.dargs);
-    phase_mark(pl, st, 0);
-    k_x_b<<<nb, kThreads, kRingBSmem, st>>>(pl.dargs);
-    phase_mark(pl, st, 1);
-    k_x_res<<<nb, kThreads, 0, st>>>(pl.dargs, 0);
-    phase_mark(pl, st, 2);
-    if ((e = fcg_precond(pl, kind, st, fd, false, 1)) != cudaSuccess) return e;
-    phase_mark(pl, st, 3);
-    if ((e = fcg_precond(pl, kind, st, fd, false, 2)) != cudaSuccess) return e;
-    phase_mark(pl, st, 5);
-    if (!fd) {
-      k_x_dots<<<nb, kThreads, 0, st>>>(pl.dargs, 0);
-      phase_mark(pl, st, 4);
-    }
-  }
-  k_x_fold<<<nb, kThreads, 0, st>>>(pl.dargs);
-  return cudaGetLastError();
-}
-
-static cudaError_t fcg_eager(Plan& pl, int kind, cudaStream_t st) {
-  if (mixed_fcg(pl, kind)) return fcg_eager_mixed(pl, kind, st);
-  const MapDesc& M = pl.hmaps[0];
-  const int nb = tile_blocks(pl);
-  cudaError_t e = fcg_attrs();
-  if (e != cudaSuccess) return e;
-  phase_mark(pl, st, -1);
-  k_f_res<<<nb, kThreads, 0, st>>>(pl.dargs, 0);
-  phase_mark(pl, st, 2);
-  if (kind == ULP_PRECOND_DCT) e = dct_prepare_mask(*pl.dct, M.f.mask, M.pitch, st);
-  if (e == cudaSuccess && kind == ULP_PRECOND_MG) e = mg_setup(*pl.mg, pl.dstate, st);
-  if (e == cudaSuccess) e = rb_setup(pl, kind, pl.dstate, st);
-  if (e == cudaSuccess) e = fcg_precond(pl, kind, st);
-  if (e != cudaSuccess) return e;
-  phase_mark(pl, st, 3);
-  k_f_dots<<<nb, kThreads, 0, st>>>(pl.dargs, 1);
+  if (!fd) k_x_dots<<<nb, kThreads, 0, st>>>(f, 1);
+  fcg_finish(pl, kind, f, fd, true, st);
   phase_mark(pl, st, 4);
   for (long long l = 0;; ++l) {
     int done = 0;
@@ -799,26 +854,67 @@ static cudaError_t fcg_eager(Plan& pl, int kind, cudaStream_t st) {
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
     if (done || l > (1LL << 24)) break;
     phase_mark(pl, st, -1);
-    k_f_a<<<nb, kThreads, 0, st>>>(pl.dargs);
+    k_x_a<<<nb, kThreads, 0, st>>>(f);
     phase_mark(pl, st, 0);
-    k_f_b<<<nb, kThreads, kRingFSmem, st>>>(pl.dargs);
+    k_x_b<<<nb, kThreads, kRingBSmem, st>>>(f);
     phase_mark(pl, st, 1);
-    k_f_res<<<nb, kThreads, 0, st>>>(pl.dargs, 1);
+    k_x_res<<<nb, kThreads, 0, st>>>(f, 0);
+    phase_mark(pl, st, 2);
+    if ((e = fcg_precond(pl, kind, f, st, fd, 1)) != cudaSuccess) return e;
+    phase_mark(pl, st, 3);
+    if ((e = fcg_precond(pl, kind, f, st, fd, 2)) != cudaSuccess) return e;
+    phase_mark(pl, st, 5);
+    if (!fd) k_x_dots<<<nb, kThreads, 0, st>>>(f, 0);
+    fcg_finish(pl, kind, f, fd, false, st);
+    phase_mark(pl, st, 4);
+  }
+  k_x_fold<<<nb, kThreads, 0, st>>>(f);
+  return cudaGetLastError();
+}
+
+static cudaError_t fcg_eager(Plan& pl, int kind, const FcgArgs& f, cudaStream_t st) {
+  if (mixed_fcg(pl, kind)) return fcg_eager_mixed(pl, kind, f, st);
+  const MapDesc& M = pl.hmaps[0];
+  const int nb = tile_blocks(pl);
+  cudaError_t e = fcg_attrs();
+  if (e != cudaSuccess) return e;
+  phase_mark(pl, st, -1);
+  k_f_res<<<nb, kThreads, 0, st>>>(f, 0);
+  phase_mark(pl, st, 2);
+  if (kind == ULP_PRECOND_DCT) e = dct_prepare_mask(*pl.dct, M.f.mask, M.pitch, st);
+  if (e == cudaSuccess && kind == ULP_PRECOND_MG) e = mg_setup(*pl.mg, pl.dstate, st);
+  if (e == cudaSuccess) e = rb_setup(pl, kind, pl.dstate, st);
+  if (e == cudaSuccess) e = fcg_precond(pl, kind, f, st);
+  if (e != cudaSuccess) return e;
+  phase_mark(pl, st, 3);
+  k_f_dots<<<nb, kThreads, 0, st>>>(f, 1);
+  fcg_finish(pl, kind, f, false, true, st);
+  phase_mark(pl, st, 4);
+  for (long long l = 0;; ++l) {
+    int done = 0;
+    if ((e = cudaMemcpyAsync(&done, &pl.dstate->done, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+    if (done || l > (1LL << 24)) break;
+    phase_mark(pl, st, -1);
+    k_f_a<<<nb, kThreads, 0, st>>>(f);
+    phase_mark(pl, st, 0);
+    k_f_b<<<nb, kThreads, kRingFSmem, st>>>(f);
+    phase_mark(pl, st, 1);
+    k_f_res<<<nb, kThreads, 0, st>>>(f, 1);
     phase_mark(pl, st, 2);
     const bool fd = fused_dots(pl, kind);
     if (kind == ULP_PRECOND_MG) {
-      if ((e = fcg_precond(pl, kind, st, fd, false, 1)) != cudaSuccess) return e;
+      if ((e = fcg_precond(pl, kind, f, st, fd, 1)) != cudaSuccess) return e;
       phase_mark(pl, st, 3);
-      if ((e = fcg_precond(pl, kind, st, fd, false, 2)) != cudaSuccess) return e;
+      if ((e = fcg_precond(pl, kind, f, st, fd, 2)) != cudaSuccess) return e;
       phase_mark(pl, st, 5);
     } else {
-      if ((e = fcg_precond(pl, kind, st, fd)) != cudaSuccess) return e;
+      if ((e = fcg_precond(pl, kind, f, st, fd)) != cudaSuccess) return e;
       phase_mark(pl, st, 3);
     }
-    if (!fd) {
-      k_f_dots<<<nb, kThreads, 0, st>>>(pl.dargs, 0);
-      phase_mark(pl, st, 4);
-    }
+    if (!fd) k_f_dots<<<nb, kThreads, 0, st>>>(f, 0);
+    fcg_finish(pl, kind, f, fd, false, st);
+    phase_mark(pl, st, 4);
   }
   return cudaGetLastError();
 }
@@ -842,22 +938,22 @@ cudaError_t launch_fcg(Plan& pl, int kind, const PcgArgs& a_in, cudaStream_t st,
   a.xfcg = mixed_fcg(pl, kind);
   if (kind == ULP_PRECOND_MG && !a.xfcg) a.rf32 = mg_input(*pl.mg);
   a.learned = kind == ULP_PRECOND_LEARNED;
+  a.cond = 0;
+  const FcgArgs f{a, pl.hmaps[0], pl.dargs};
   if (pl.opt.profile == 2) {
-    a.cond = 0;
     k_set_args<<<1, 1, 0, st>>>(a, pl.dargs);
     launch_pcg_reset(pl, st);
     if (e0) cudaEventRecord(e0, st);
-    const cudaError_t e = fcg_eager(pl, kind, st);
+    const cudaError_t e = fcg_eager(pl, kind, f, st);
     if (e == cudaSuccess && e1) cudaEventRecord(e1, st);
     return e;
   }
   if (pl.fcg_exec && (pl.fcg_kind != kind || (kind == ULP_PRECOND_LEARNED && pl.fcg_gen != unet_ws_gen(*pl.unet))))
     destroy_fcg(pl);
   if (!pl.fcg_exec) {
-    const cudaError_t e = fcg_build(pl, kind);
+    const cudaError_t e = fcg_build(pl, kind, f);
     if (e != cudaSuccess) return e;
   }
-  a.cond = pl.fcg_cond;
   pl.kernel_launches += 2;
   pl.solver_launches += 1;
   k_set_args<<<1, 1, 0, st>>>(a, pl.dargs);

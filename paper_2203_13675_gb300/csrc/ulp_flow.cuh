@@ -95,26 +95,21 @@ __device__ __forceinline__ void flow_publish(const PcgArgs& a, const FlowMap& L,
   }
 }
 
-// Sum of one array of n tile partials by 128 threads (r = 0 .. 127), into part[32]: tile i
-// belongs to group i mod 32; within a group, lane l of 32 adds tiles l, l + 32, ... of the
-// group in order and the lanes add up as a shuffle-down tree (16, 8, 4, 2, 1) -- the order
-// of tile_arrive, so both give the same bits.  A thread holds lanes c, c + 4, ..., c + 28 of
-// its group: the tree's first three levels stay in registers, where an FP64 add of a warp
-// costs its 64 cycles for 32 useful lanes instead of for a few.
+// group_sums of slots that may still hold the sentinel; false if the wait ran out.
 __device__ __forceinline__ bool flow_group_sums(const double* P, int n, int r, double* part,
                                                 unsigned long long timeout_ns, int* err) {
-  const int g = ((r >> 5) << 3) + (r & 7), c = (r & 31) >> 3;
+  const GroupLane t(r);
   double acc[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) acc[q] = 0.0;
   bool ok = true;
   unsigned long long t_start = 0;
-  for (int k = 0; g + kArriveGroups * (c + 32 * k) < n; ++k) {
+  for (int k = 0; t.first(k) < n; ++k) {
     double v[8];
     bool again = false;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const int i = g + kArriveGroups * (c + 4 * q + 32 * k);
+      const int i = t.first(k) + 4 * kArriveGroups * q;
       v[q] = i < n ? ld_relaxed(P + i) : 0.0;
     }
 #pragma unroll
@@ -125,7 +120,7 @@ __device__ __forceinline__ bool flow_group_sums(const double* P, int n, int r, d
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         if (is_sentinel(v[q])) {
-          v[q] = ld_relaxed(P + g + kArriveGroups * (c + 4 * q + 32 * k));
+          v[q] = ld_relaxed(P + t.first(k) + 4 * kArriveGroups * q);
           again |= is_sentinel(v[q]);
         }
       }
@@ -139,14 +134,7 @@ __device__ __forceinline__ bool flow_group_sums(const double* P, int n, int r, d
 #pragma unroll
     for (int q = 0; q < 8; ++q) acc[q] += v[q];
   }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) acc[q] += acc[q + 4];
-  acc[0] += acc[2];
-  acc[1] += acc[3];
-  double s = acc[0] + acc[1];
-  s += __shfl_down_sync(kFull, s, 16);  // lanes c + 2 of the group
-  s += __shfl_down_sync(kFull, s, 8);   // lanes c + 1
-  if (c == 0) part[g] = s;
+  group_tree(t, acc, part);
   return ok;
 }
 

@@ -40,7 +40,6 @@ struct Plan {
   void* dct_mem = nullptr;
   PcgArgs* dargs = nullptr;  // solver arguments in device memory (read by the graph-driven solve)
   cudaGraphExec_t fcg_exec = nullptr;       // flexible-CG solve graph (DCT preconditioner)
-  unsigned long long fcg_cond = 0;          // its WHILE-node handle
   int fcg_kind = -1;                        // preconditioner the flexible-CG graph was built for
   long long fcg_start_kernels = 0;          // kernels of its start and of one WHILE-body execution
   long long fcg_body_kernels = 0;
@@ -120,22 +119,22 @@ int dct_error(const DctPlan& d);  // 1 if a GEMM wait ran out since the last cal
 // ulp_fcg.cu
 // ulp_mg.cu: aggregation multigrid on the map's planes (U, V, D^-1; r -> s, y as scratch)
 size_t mg_bytes(int H, int W);
-MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles);
+// max_units: partials of the map grid's last kernel that the plan has room for
+MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles, int max_units);
 void mg_destroy(MgPlan* p);
 // coarse grids, once per solve; level0: make the map grid's FP32 weights and D^-1 from the FP64
 // planes (false when launch_system_x already wrote them)
 cudaError_t mg_setup(const MgPlan& p, const MapState* S, cudaStream_t st, bool level0 = true);
-// packed: the FP32 copy of r (mg_input, the map's pitch) is already written; dots (device
-// arguments of a flexible-CG solve, or null): the cycle's last kernel also does the solve's
-// dot phase (r^T s, r^T r, beta, stop test), if mg_fuses_dots
+// packed: the FP32 copy of r (mg_input, the map's pitch) is already written; dots (a flexible-CG
+// solve's arguments, or null): the cycle's last kernel also leaves the partials
+// of r^T s (and, in FP64, r^T r), if mg_fuses_dots
 // s32 (or null): s is written in FP32 there instead of the map's FP64 s plane (the mixed flexible CG)
-// dots_init: the dot phase is the start of a solve (r^T s, r^T r, and b^T b from the
-// per-tile partials that k_x_res left in P2)
 // part: 0 the whole cycle; 1 all but its last kernel (the up step on the map's grid); 2 that
 // last kernel alone (the host-driven replay times it on its own)
 cudaError_t mg_apply(const MgPlan& p, const uint8_t* mask, const MapState* S, cudaStream_t st, bool packed = false,
-                     const PcgArgs* dots = nullptr, float* s32 = nullptr, bool dots_init = false, int part = 0);
+                     const PcgArgs* dots = nullptr, float* s32 = nullptr, int part = 0);
 bool mg_fuses_dots(const MgPlan& p);
+int mg_dot_units(const MgPlan& p);  // partials of the fused dot phase
 float* mg_input(const MgPlan& p);
 int mg_levels(const MgPlan& p);
 

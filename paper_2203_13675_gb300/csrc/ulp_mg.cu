@@ -528,15 +528,25 @@ __global__ void __launch_bounds__(kTileThreads) k_mg_down_t(Grid f, Grid c, int 
 
 // prolongation + correction + both post-sweeps for the rows [TR band, TR band + TR).
 // xc: the coarse grid's corrected solution.  MODE kUpCoarse: s to the grid's t plane.
-// kUp64 (the map's grid): s in FP64; with pa, r^T s and r^T r (r: the map's FP64
+// kUp64 (the map's grid): s in FP64; with dp0, r^T s and r^T r (r: the map's FP64
 // residual) over the block's pixels arrive in the flexible CG's dot phase.  kUp32 (the
-// map's grid, mixed flexible CG): s in FP32 into s32; with pa, the same dot phase in
+// map's grid, mixed flexible CG): s in FP32 into s32; with dp0, the same dot phase in
 // double-float sums of exact FP32 products, r being the cycle's right-hand side.
 enum { kUpCoarse = 0, kUp64 = 1, kUp32 = 2 };
+// The partials of unit w (a warp or a block) of the flexible CG's dot phase.
+template <int MODE>
+__device__ __forceinline__ void dot_partials(double* dp0, double* dp1, int w, double rs, double rr, int lane) {
+  rs = warp_sum(rs);
+  if (MODE == kUp64) rr = warp_sum(rr);  // mixed: r^T r comes per tile
+  if (lane == 0) {
+    __stcg(dp0 + w, rs);
+    if (MODE == kUp64) __stcg(dp1 + w, rr);
+  }
+}
 template <int MODE>
 __global__ void __launch_bounds__(kTileThreads) k_mg_up_t(Grid f, Grid c, const float* __restrict__ xc, int TR,
                                                         const uint8_t* mask, double* s, const double* __restrict__ rv,
-                                                        float* s32, const PcgArgs* pa, const MapState* S, int ph) {
+                                                        float* s32, double* const dp0, double* const dp1, const MapState* S) {
   constexpr bool MAP = MODE != kUpCoarse;
   constexpr int kOut = kTileMaxRows / kTileWarps;  // output rows per warp at most
   if (skip_map(S)) return;
@@ -623,7 +633,7 @@ __global__ void __launch_bounds__(kTileThreads) k_mg_up_t(Grid f, Grid c, const 
       const float4 sv = make_float4(mk[k].x ? 0.f : v.x, mk[k].y ? 0.f : v.y, mk[k].z ? 0.f : v.z,
                                     mk[k].w ? 0.f : v.w);
       *reinterpret_cast<float4*>(s32 + o) = sv;
-      if (pa) {
+      if (dp0) {
         // r is the cycle's right-hand side (zero beyond column W - 1, as is s there);
         // r^T r comes per tile from the kernels that wrote r
         rs32.add_prod(B.x, sv.x);
@@ -643,7 +653,7 @@ __global__ void __launch_bounds__(kTileThreads) k_mg_up_t(Grid f, Grid c, const 
         for (int q = 0; q < 4; ++q)
           if (j + q < f.W) s[o + q] = sv[q];
       }
-      if (pa && rv) {
+      if (dp0 && rv) {
         const double rk[4] = {ra[k].x, ra[k].y, rb[k].x, rb[k].y};
 #pragma unroll
         for (int q = 0; q < 4; ++q)
@@ -654,9 +664,9 @@ __global__ void __launch_bounds__(kTileThreads) k_mg_up_t(Grid f, Grid c, const 
       }
     }
   }
-  if (MAP && pa) {
+  if (MAP && dp0) {
     if (MODE == kUp32) rs = rs32.value();
-    // block sums in warp order, then the arrival of the block as one unit
+    // block sums in warp order, then the block's partials as one unit
     rs = warp_sum(rs);
     rr2 = warp_sum(rr2);
     if (lane == 0) {
@@ -665,9 +675,8 @@ __global__ void __launch_bounds__(kTileThreads) k_mg_up_t(Grid f, Grid c, const 
     }
     __syncthreads();
     if (warp == 0) {
-      const PcgArgs a = *pa;
       const double v0 = lane < kTileWarps ? red[0][lane] : 0.0, v1 = lane < kTileWarps ? red[1][lane] : 0.0;
-      warp_arrive_fcg(a, a.maps[0], a.st, (int)blockIdx.x, (int)gridDim.x, v0, v1, lane, ph, MODE == kUp32);
+      dot_partials<MODE>(dp0, dp1, (int)blockIdx.x, v0, v1, lane);
     }
   }
 }
@@ -835,7 +844,7 @@ template <int MODE>
 __global__ void __launch_bounds__(kWalkWarps * 32) k_mg_up_w(Grid f, Grid c, const float* __restrict__ xc, int R,
                                                              const uint8_t* mask, double* s,
                                                              const double* __restrict__ rv, float* s32,
-                                                             const PcgArgs* pa, const MapState* S, int ph) {
+                                                             double* const dp0, double* const dp1, const MapState* S) {
   constexpr bool MAP = MODE != kUpCoarse;
   if (skip_map(S)) return;
   extern __shared__ float4 wsm4[];
@@ -886,7 +895,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32) k_mg_up_w(Grid f, Grid c, con
         if (MODE == kUp32) {
           const float4 sv = make_float4(mk.x ? 0.f : v.x, mk.y ? 0.f : v.y, mk.z ? 0.f : v.z, mk.w ? 0.f : v.w);
           *reinterpret_cast<float4*>(s32 + o) = sv;
-          if (pa) {
+          if (dp0) {
             // r is the cycle's right-hand side (zero beyond column W - 1, as is s there);
             // r^T r comes per tile from the kernels that wrote r
             rs32.add_prod(Bm2.x, sv.x);
@@ -926,11 +935,10 @@ __global__ void __launch_bounds__(kWalkWarps * 32) k_mg_up_w(Grid f, Grid c, con
     XPm2 = XPm1; XPm1 = XP;
     Tm3 = Tm2; Tm2 = T;
   }
-  if (MAP && pa) {
-    const PcgArgs a = *pa;
+  if (MAP && dp0) {
     const int nseg = (f.W + kSegOut - 1) / kSegOut;
     if (MODE == kUp32) rs = rs32.value();
-    warp_arrive_fcg(a, a.maps[0], a.st, band * nseg + seg, nseg * bands, rs, rr, lane, ph, MODE == kUp32);
+    dot_partials<MODE>(dp0, dp1, band * nseg + seg, rs, rr, lane);
   }
 }
 
@@ -1232,7 +1240,7 @@ static unsigned tile_blocks(const Grid& f, int TR) {
   return (unsigned)(((f.W + kSegOut - 1) / kSegOut) * ((f.H + TR - 1) / TR));
 }
 
-MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles) {
+MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles, int max_units) {
   MgPlan* p = new MgPlan();
   p->mem = mem;
   p->nsm = nsm;
@@ -1325,7 +1333,8 @@ MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles) {
     const long long n = p->kind[0] == kWalk
                             ? (long long)((M.W + kSegOut - 1) / kSegOut) * ((M.H + p->rows_up[0] - 1) / p->rows_up[0])
                             : (long long)tile_blocks(p->g[0], p->rows_up[0]);
-    if (n >= kArriveGroups && n <= ntiles) p->dots_units = (int)n;
+    // (FP64 plans, max_units = ntiles: not on the smallest maps, whose sums keep the tiles' order)
+    if (n <= max_units && (n >= kArriveGroups || max_units > ntiles)) p->dots_units = (int)n;
   }
 
   // the tail: the smallest suffix of grids, from the first with at most kTailMax unknowns,
@@ -1354,6 +1363,7 @@ MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles) {
 void mg_destroy(MgPlan* p) { delete p; }
 
 bool mg_fuses_dots(const MgPlan& p) { return p.dots_units > 0; }
+int mg_dot_units(const MgPlan& p) { return p.dots_units; }
 
 static unsigned row_blocks(const Grid& f, int rows) {
   const long long warps = (long long)rows * ((f.W + 127) / 128);
@@ -1393,9 +1403,9 @@ cudaError_t mg_setup(const MgPlan& p, const MapState* S, cudaStream_t st, bool l
 float* mg_input(const MgPlan& p) { return p.g[0].b; }
 
 // The up step of grid l; on the map's grid (l = 0) it writes s (FP64, or FP32 into
-// s32) and, with dots, carries the flexible CG's dot phase ph.
+// s32) and, with dots, makes the flexible CG's dot partials.
 static void up_level(const MgPlan& p, int l, int stop, const uint8_t* mask, const MapState* S, cudaStream_t st,
-                     const PcgArgs* dots, float* s32, int ph) {
+                     const PcgArgs* dots, float* s32) {
   const Grid& f = p.g[l];
   if (p.kind[l] != kPerStep) {
     // the coarse grid's corrected solution: the t plane if a fused kernel made it, else x
@@ -1403,7 +1413,6 @@ static void up_level(const MgPlan& p, int l, int stop, const uint8_t* mask, cons
     const float* xc = (l + 1 < stop && p.kind[l + 1] != kPerStep) ? c.t : c.x;
     const int R = p.rows_up[l];
     const bool d = l == 0 && dots && p.dots_units > 0;
-    const PcgArgs* pa = d ? dots : nullptr;
     const int mode = l > 0 ? kUpCoarse : (s32 ? kUp32 : kUp64);
     const double* rv = (mode == kUp64 && d) ? p.r0 : nullptr;
     double* s64 = mode == kUp64 ? p.s0 : nullptr;
@@ -1412,14 +1421,14 @@ static void up_level(const MgPlan& p, int l, int stop, const uint8_t* mask, cons
     if (p.kind[l] == kWalk) {
       const unsigned nb = walk_blocks(f, f.H, R);
       const unsigned nt = kWalkWarps * 32;
-      if (mode == kUp32) k_mg_up_w<kUp32><<<nb, nt, kUpRingSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, pa, S, ph);
-      else if (mode == kUp64) k_mg_up_w<kUp64><<<nb, nt, kUpRingSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, pa, S, ph);
-      else k_mg_up_w<kUpCoarse><<<nb, nt, kUpRingSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, pa, S, ph);
+      if (mode == kUp32) k_mg_up_w<kUp32><<<nb, nt, kUpRingSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
+      else if (mode == kUp64) k_mg_up_w<kUp64><<<nb, nt, kUpRingSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
+      else k_mg_up_w<kUpCoarse><<<nb, nt, kUpRingSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
     } else {
       const unsigned nb = tile_blocks(f, R);
-      if (mode == kUp32) k_mg_up_t<kUp32><<<nb, kTileThreads, kTileSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, pa, S, ph);
-      else if (mode == kUp64) k_mg_up_t<kUp64><<<nb, kTileThreads, kTileSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, pa, S, ph);
-      else k_mg_up_t<kUpCoarse><<<nb, kTileThreads, kTileSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, pa, S, ph);
+      if (mode == kUp32) k_mg_up_t<kUp32><<<nb, kTileThreads, kTileSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
+      else if (mode == kUp64) k_mg_up_t<kUp64><<<nb, kTileThreads, kTileSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
+      else k_mg_up_t<kUpCoarse><<<nb, kTileThreads, kTileSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
     }
     return;
   }
@@ -1437,8 +1446,7 @@ static void up_level(const MgPlan& p, int l, int stop, const uint8_t* mask, cons
 }
 
 cudaError_t mg_apply(const MgPlan& p, const uint8_t* mask, const MapState* S, cudaStream_t st, bool packed,
-                     const PcgArgs* dots, float* s32, bool dots_init, int part) {
-  const int ph = dots_init ? kPhResInit : kPhFcg;
+                     const PcgArgs* dots, float* s32, int part) {
   const int L = (int)p.g.size();
   const Grid& g0 = p.g[0];
   const int stop = p.lt > 0 ? p.lt : L - 1;  // grids [0, stop) by per-grid kernels
@@ -1448,7 +1456,7 @@ cudaError_t mg_apply(const MgPlan& p, const uint8_t* mask, const MapState* S, cu
       k_mg_post2<<<mg_blocks(p, (long long)g0.H * g0.W), 256, 0, st>>>(g0, mask, p.s0, S);
       if (s32) k_mg_to32<<<mg_blocks(p, (long long)g0.H * g0.W), 256, 0, st>>>(p.s0, s32, g0, S);
     } else {
-      up_level(p, 0, stop, mask, S, st, dots, s32, ph);
+      up_level(p, 0, stop, mask, S, st, dots, s32);
     }
     return cudaGetLastError();
   }
@@ -1482,7 +1490,7 @@ cudaError_t mg_apply(const MgPlan& p, const uint8_t* mask, const MapState* S, cu
   } else {
     k_mg_coarsest<<<1, 256, 0, st>>>(p.g[L - 1], S);
   }
-  for (int l = stop - 1; l >= (part == 1 ? 1 : 0); --l) up_level(p, l, stop, mask, S, st, dots, s32, ph);
+  for (int l = stop - 1; l >= (part == 1 ? 1 : 0); --l) up_level(p, l, stop, mask, S, st, dots, s32);
   return cudaGetLastError();
 }
 

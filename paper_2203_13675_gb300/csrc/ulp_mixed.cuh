@@ -198,12 +198,5 @@ __device__ __forceinline__ double a32_tile_dq(const PcgArgs& a, const MapDesc& M
   stencil_tile32(M, g.i0, g.i1, g.j0, lane, M.h.U, M.h.V, x, epi, ring);
   return dq.value();
 }
-// The same as phase A of a solve whose scalars live in the map's state.
-template <int KIND>
-__device__ __forceinline__ void a32_tile(const PcgArgs& a, const MapDesc& M, MapState* S, int t, int lane,
-                                         Slot32* ring) {
-  const double dq = a32_tile_dq<KIND>(a, M, t, *(volatile long long*)&S->iter, *(volatile double*)&S->beta, lane, ring);
-  tile_arrive(a, M, S, t, kPhA, dq, 0.0, 0.0, lane);
-}
 
 }  // namespace ulp
