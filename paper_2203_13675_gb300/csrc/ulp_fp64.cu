@@ -26,7 +26,7 @@ __global__ void k_pack(MapDesc M, MapState* S, const double* __restrict__ psi,
     if (j < M.W) {
       const size_t k = (size_t)i * M.W + j;
       const double c = psi[k];
-      if (!isfinite(c)) atomicExch(&S->err_flag, 1);
+      if (((unsigned)__double2hiint(c) & 0x7ff00000u) == 0x7ff00000u) atomicExch(&S->err_flag, 1);  // not finite
       if (j + 1 < M.W) dx = wrap_pv(__dsub_rn(psi[k + 1], c));
       if (i + 1 < M.H) dy = wrap_pv(__dsub_rn(psi[k + M.W], c));
       if (mask) mk = mask[k] ? 1 : 0;
@@ -171,8 +171,13 @@ __global__ void k_weights_x(const MapDesc* __restrict__ maps, MapState* S, const
     }
     *reinterpret_cast<float2*>(M.h.U + o) = u;
     *reinterpret_cast<float2*>(M.h.V + o) = v;
-    st2(M.f.U, o, make_double2((double)u.x, (double)u.y));
-    st2(M.f.V, o, make_double2((double)v.x, (double)v.y));
+    if (is_plain(u.x) && is_plain(u.y) && is_plain(v.x) && is_plain(v.y)) {
+      st2(M.f.U, o, make_double2(widen_plain(u.x), widen_plain(u.y)));
+      st2(M.f.V, o, make_double2(widen_plain(v.x), widen_plain(v.y)));
+    } else {  // weights below FP32's normal range
+      st2(M.f.U, o, make_double2((double)u.x, (double)u.y));
+      st2(M.f.V, o, make_double2((double)v.x, (double)v.y));
+    }
     st2(M.f.phi_prev, o, ph);
   }
 }
@@ -211,7 +216,9 @@ __global__ void k_system_x(const MapDesc* __restrict__ maps, MapState* S) {
       bk = __fma_rn(-dyv2[k], vsv[k], bk);
       d2[k] = d;
       b2[k] = bk;
-      di[k] = (d > 0.0) ? __fdiv_rn(1.f, (float)d) : 0.f;
+      // (a sum of FP32 weights: positive in FP64 is positive in FP32)
+      const float df = (float)d;
+      di[k] = (df > 0.f) ? __fdiv_rn(1.f, df) : 0.f;
     }
     st2(M.f.D, o, make_double2(d2[0], d2[1]));
     st2(M.f.b, o, make_double2(b2[0], b2[1]));
