@@ -453,23 +453,34 @@ __global__ void __launch_bounds__(256) k_dir_stats(Src s, Offs ro, Offs uo, cons
   }
 }
 
-// per image: coefficients c1, c2 (scaled by 1/B) into coef[2b], coef[2b+1]; the batch loss
-__global__ void k_dir_reduce(const double* __restrict__ part, int nb, int B, double* __restrict__ coef,
-                             double* __restrict__ loss) {
-  if (threadIdx.x != 0) return;
-  double L = 0.0;
-  for (int b = 0; b < B; ++b) {
+// per image: coefficients c1, c2 (scaled by 1/B) into coef[2b], coef[2b+1]; the batch loss.
+// One block, a warp per image in turn: the partials of its three sums over the lanes, then a
+// tree (one thread adding 3 x 64 x B partials one load after the other took 102 us at B = 8).
+__global__ void __launch_bounds__(1024) k_dir_reduce(const double* __restrict__ part, int nb, int B,
+                                                     double* __restrict__ coef, double* __restrict__ loss) {
+  __shared__ double sl[kMaxBatch];
+  const int lane = threadIdx.x & 31;
+  for (int b = threadIdx.x >> 5; b < B; b += 32) {
     double a = 0.0, bb = 0.0, g = 0.0;
-    for (int k = 0; k < nb; ++k) {
+    for (int k = lane; k < nb; k += 32) {
       a += part[((size_t)b * nb + k) * 3 + 0];
       bb += part[((size_t)b * nb + k) * 3 + 1];
       g += part[((size_t)b * nb + k) * 3 + 2];
     }
-    const bool ok = bb > 0.0 && g > 0.0;
-    coef[2 * b] = ok ? -2.0 * a / (bb * g) / B : 0.0;
-    coef[2 * b + 1] = ok ? 2.0 * a * a / (bb * bb * g) / B : 0.0;
-    L += ok ? 1.0 - a * a / (bb * g) : 1.0;
+    a = warp_sum(a);
+    bb = warp_sum(bb);
+    g = warp_sum(g);
+    if (lane == 0) {
+      const bool ok = bb > 0.0 && g > 0.0;
+      coef[2 * b] = ok ? -2.0 * a / (bb * g) / B : 0.0;
+      coef[2 * b + 1] = ok ? 2.0 * a * a / (bb * bb * g) / B : 0.0;
+      sl[b] = ok ? 1.0 - a * a / (bb * g) : 1.0;
+    }
   }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  double L = 0.0;
+  for (int b = 0; b < B; ++b) L += sl[b];
   *loss = L / B;
 }
 
@@ -542,19 +553,32 @@ __global__ void __launch_bounds__(256) k_head_train(const bf16* __restrict__ g0,
   GRID_STRIDE(q, n) {
     float f[16];
     head_dot(g0 + q * 16, hw, 0.f, f);
-    const double d = (double)dyp[q];
+    // FP64 only for the sums (exact products): the conversions and the FP32 products on the FP64
+    // pipe as well made this 182 us for eight 512x512 images, now HEAD_FIGURE
+    const float dy = dyp[q];
+    bool plain = is_plain(dy);
+#pragma unroll
+    for (int c = 0; c < 16; ++c) plain &= is_plain(f[c]);
     float o0[8], o1[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-      o0[c] = f[c] > 0.f ? (float)(d * hw[c]) : 0.f;
-      o1[c] = f[8 + c] > 0.f ? (float)(d * hw[8 + c]) : 0.f;
+      o0[c] = f[c] > 0.f ? __fmul_rn(dy, hw[c]) : 0.f;
+      o1[c] = f[8 + c] > 0.f ? __fmul_rn(dy, hw[8 + c]) : 0.f;
     }
     uint4* dst = reinterpret_cast<uint4*>(dg0 + q * 16);
     dst[0] = pack8(o0);
     dst[1] = pack8(o1);
+    if (plain) {
+      const double d = widen_plain(dy);
 #pragma unroll
-    for (int c = 0; c < 16; ++c) acc[c] += d * (double)f[c];
-    acc[16] += d;
+      for (int c = 0; c < 16; ++c) acc[c] = fma(d, widen_plain(f[c]), acc[c]);
+      acc[16] += d;
+    } else {
+      const double d = (double)dy;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) acc[c] = fma(d, (double)f[c], acc[c]);
+      acc[16] += d;
+    }
   }
   __shared__ double sh[8][17];
 #pragma unroll
@@ -569,12 +593,12 @@ __global__ void __launch_bounds__(256) k_head_train(const bf16* __restrict__ g0,
     part[(size_t)blockIdx.x * 17 + threadIdx.x] = s;
   }
 }
+// One warp per sum (17 threads adding nb partials one load after the other: 43 us).
 __global__ void k_head_reduce(const double* __restrict__ part, int nb, float* __restrict__ ghead) {
-  const int k = threadIdx.x;
-  if (k >= 17) return;
   double s = 0.0;
-  for (int b = 0; b < nb; ++b) s += part[(size_t)b * 17 + k];
-  ghead[k] = (float)s;
+  for (int b = threadIdx.x; b < nb; b += 32) s += part[(size_t)b * 17 + blockIdx.x];
+  s = warp_sum(s);
+  if (threadIdx.x == 0) ghead[blockIdx.x] = (float)s;
 }
 
 // ------------------------------------------------------------------ weight gradient
@@ -829,16 +853,46 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(WgArgs a) {
 // canonical gradient of one layer: W [O][C][3][3] at gw, bias [O] at gb; sums the
 // splits of part[split][m][o] (m = c 9 + t, the bias row at m = 9 C) in order.  Thread e
 // takes (m, o) = (e / O, e mod O), so a warp reads consecutive o of one row.
-__global__ void k_wgrad_reduce(const float* __restrict__ part, int nsplit, int mtiles, int O, int C,
-                               float* __restrict__ gw, float* __restrict__ gb) {
+// A block adds 32 elements' splits: thread (element, slice) takes every SL-th split, its loads in
+// flight together, then the slices as a tree (one thread per element adding 41 to 607 splits in
+// turn took 34 to 111 us a layer).  Many splits come with few elements, so those take more slices.
+template <int SL>
+__global__ void __launch_bounds__(32 * SL) k_wgrad_reduce(const float* __restrict__ part, int nsplit, int mtiles, int O,
+                                                          int C, float* __restrict__ gw, float* __restrict__ gb) {
+  __shared__ double sh[SL][32];
   const int n = (9 * C + 1) * O;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-    const int m = e / O, o = e - m * O;
-    double s = 0.0;
-    for (int g = 0; g < nsplit; ++g) s += part[((size_t)g * mtiles * 128 + m) * O + o];
-    if (m < 9 * C) gw[(size_t)o * 9 * C + m] = (float)s;  // W[o][c][t] at o 9 C + c 9 + t
-    else gb[o] = (float)s;
+  const int el = threadIdx.x & 31, sl = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + el;
+  const int m = e / O, o = e - m * O;
+  double s = 0.0;
+  if (e < n) {
+    const float* p = part + (size_t)m * O + o;
+    const size_t step = (size_t)mtiles * 128 * O;
+    for (int g0 = sl; g0 < nsplit; g0 += 8 * SL) {
+      float v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = g0 + k * SL < nsplit ? __ldg(p + (size_t)(g0 + k * SL) * step) : 0.f;
+      bool plain = true;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) plain &= is_plain(v[k]);
+      if (plain) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s += widen_plain(v[k]);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s += (double)v[k];
+      }
+    }
   }
+  sh[sl][el] = s;
+#pragma unroll
+  for (int h = SL / 2; h > 0; h >>= 1) {
+    __syncthreads();
+    if (sl < h) sh[sl][el] = s = s + sh[sl + h][el];
+  }
+  if (sl != 0 || e >= n) return;
+  if (m < 9 * C) gw[(size_t)o * 9 * C + m] = (float)s;  // W[o][c][t] at o 9 C + c 9 + t
+  else gb[o] = (float)s;
 }
 
 // once per device, before any capture
@@ -1065,7 +1119,9 @@ static cudaError_t wgrad(Unet& u, int l, const bf16* dy, const bf16* x, int Cx, 
     default: return cudaErrorInvalidValue;
   }
   const int n = (9 * a.C + 1) * a.O;
-  k_wgrad_reduce<<<(n + 255) / 256, 256, 0, st>>>(u.part, (int)nsplit, a.mtiles, a.O, a.C, u.grad + u.off.w[l],
+  if (nsplit > 128) k_wgrad_reduce<32><<<(n + 31) / 32, 1024, 0, st>>>(u.part, (int)nsplit, a.mtiles, a.O, a.C, u.grad + u.off.w[l],
+                                                  u.grad + u.off.b[l]);
+  else k_wgrad_reduce<8><<<(n + 31) / 32, 256, 0, st>>>(u.part, (int)nsplit, a.mtiles, a.O, a.C, u.grad + u.off.w[l],
                                                   u.grad + u.off.b[l]);
   return cudaGetLastError();
 }
@@ -1077,7 +1133,7 @@ static cudaError_t backward(Unet& u, int B, int Hn, int Wn, cudaStream_t st) {
   cudaError_t e;
   double* part = u.red + kRedHead;
   k_head_train<<<kHeadBlocks, 256, 0, st>>>(u.g0, u.theta + u.off.hw, u.t, n, u.dg0, part);
-  k_head_reduce<<<1, 32, 0, st>>>(part, kHeadBlocks, u.grad + u.off.hw);
+  k_head_reduce<<<17, 32, 0, st>>>(part, kHeadBlocks, u.grad + u.off.hw);
   // d0
   CK(wgrad(u, D0, u.dg0, u.cat0, 48, B, Hn, Wn, st));
   CK(conv3x3(u.dg0, B, Hn, Wn, 16, u.wb[D0], 48, nullptr, 0, u.dcat0, 48, 0, 0, nullptr, u.err, st));
@@ -1345,7 +1401,7 @@ static int loss_grad_impl(Unet& u, int B, const Offs& ro, const Offs& uo, int H,
   k_head_out<<<eblocks(n), 256, 0, st>>>(u.g0, u.theta + u.off.hw, n, u.y);
   k_dir_s<<<eblocks(n), 256, 0, st>>>(src, ro, uo, u.red + kRedRho, u.y, B, u.sd);
   k_dir_stats<<<dim3(kStatBlocks, B), 256, 0, st>>>(src, ro, uo, e, u.red + kRedRho, u.sd, u.asd, u.red + kRedDir);
-  k_dir_reduce<<<1, 32, 0, st>>>(u.red + kRedDir, kStatBlocks, B, u.red + kRedCoef, u.red + kRedLoss);
+  k_dir_reduce<<<1, B < 32 ? 32 * B : 1024, 0, st>>>(u.red + kRedDir, kStatBlocks, B, u.red + kRedCoef, u.red + kRedLoss);
   k_dir_grad<<<eblocks(n), 256, 0, st>>>(src, ro, u.red + kRedRho, u.asd, u.red + kRedCoef, B, u.t);
   UCU(backward(u, B, H, W, st));
   return ULP_OK;
