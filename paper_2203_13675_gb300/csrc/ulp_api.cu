@@ -269,7 +269,7 @@ static int plan_init(Plan& pl, int n, const int* H, const int* W, const ulp_opti
       cudaGetLastError();
       return fail(ULP_ERR_NOMEM, "cudaMalloc(DCT buffers): %s", cudaGetErrorString(e));
     }
-    pl.dct = dct_create(H[0], W[0], pl.dct_mem);
+    pl.dct = dct_create(H[0], W[0], pl.dct_mem, pl.nsm);
     if (!pl.dct) return fail(ULP_ERR_CUDA, "DCT preconditioner set-up failed");
     e = cudaMalloc(&pl.mg_mem, mg_bytes(H[0], W[0]));
     if (e != cudaSuccess) {

@@ -19,10 +19,10 @@
 // feeds the next GEMM writes both planes of its output.
 //
 // GEMM form: C[m][n] = sum_k A[m][k] B[n][k] with both operands K-major
-// (row-major, k contiguous), BM = 128, BN = 128, BK = 64 (one 128-byte
-// swizzle atom of BF16 per row), operands staged by TMA into a 3-stage ring,
-// one elected thread issuing tcgen05.mma, the accumulator read back by all
-// four warps with tcgen05.ld.  The epilogue stores C transposed, out[n][m]:
+// (row-major, k contiguous), BM = 128, BN = 128 or 64, BK = 64 (one 128-byte
+// swizzle atom of BF16 per row), operands staged by TMA into a ring,
+// one elected thread issuing tcgen05.mma, the accumulator read back by four
+// epilogue warps with tcgen05.ld.  The epilogue stores C transposed, out[n][m]:
 // a warp holds 32 consecutive m of one n, so the transposed store is the
 // coalesced one, and four transposed GEMMs chain without a transpose pass:
 //   G1  A = R (i,j)     B = C_W (b,j)    -> X^T  (b,i)
@@ -42,10 +42,19 @@
 
 namespace ulp {
 
-constexpr int kBM = 128, kBN = 128, kBK = 64, kStages = 3;
-constexpr int kTileBytes = kBM * kBK * 2;                 // 16 KB per operand tile
-constexpr int kStageBytes = 2 * kTileBytes;               // A + B
-constexpr int kGemmSmem = kStages * kStageBytes + 1024 + 256 + 512;  // + alignment + barriers + 1/Lambda rows
+constexpr int kBM = 128, kBNMax = 128, kBK = 64;
+constexpr int kTileBytes = kBM * kBK * 2;                       // 16 KB per A tile
+constexpr int stage_bytes(int BN) { return kTileBytes + BN * kBK * 2; }  // A + B
+// Tile and ring.  A block's rate is that of its operands into one SM's shared memory, 32 KB
+// per 128 x 128 x 64 step (ncu: 1.5 MB per block in about 15 us at 1024x1024, 48 bytes a clock),
+// not the tensor pipe's.  Products whose 128 x 128 tiles would leave half the SMs idle take
+// 128 x 64 tiles: twice the blocks, 24 KB a step.  Where every block has an SM to itself the
+// ring fills its shared memory; larger products run two blocks to an SM with three stages
+// each, one's epilogue under the other's main loop.  DCT_FIGURES
+constexpr int kRingBytes = 6 * stage_bytes(kBNMax);  // 192 KB: six stages at BN = 128, eight at 64
+constexpr int kStagesMany = 3;
+constexpr int kGemmThreads = 192;  // warps 0-3 epilogue, warp 4 TMA, warp 5 MMA
+constexpr int gemm_smem(int ring) { return ring + 1024 + 256 + 512; }  // + alignment + barriers + eigenvalues
 
 enum Epi { kEpiBf16T = 0, kEpiBf16TScale = 1, kEpiF64TMask = 2 };
 
@@ -61,44 +70,31 @@ struct GemmOut {
   int* err;
 };
 
-// instruction descriptor, kind::f16: D = F32, A = B = BF16, both K-major, M = 128, N = 128
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kBN >> 3) << 17) |
-                            ((uint32_t)(kBM >> 4) << 24);
-
 // tmA / tmB: the high planes, tmAl / tmBl: the low planes; K-segments (Ah, Bh), (Ah, Bl),
 // (Al, Bh) in that order, all accumulated into one tensor-memory tile
-template <int EPI>
-__global__ void __launch_bounds__(128, 1) k_gemm_nt(const __grid_constant__ CUtensorMap tmA,
+template <int EPI, int kBN>
+__global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_nt(const __grid_constant__ CUtensorMap tmA,
                                                     const __grid_constant__ CUtensorMap tmB,
                                                     const __grid_constant__ CUtensorMap tmAl,
-                                                    const __grid_constant__ CUtensorMap tmBl, int K, GemmOut o) {
+                                                    const __grid_constant__ CUtensorMap tmBl, int K, int stages,
+                                                    GemmOut o) {
+  constexpr int kStageBytes = stage_bytes(kBN);
+  constexpr uint32_t kIdesc = idesc_bf16(kBM, kBN);
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(base + kStages * kStageBytes);
-  uint64_t* empty = full + kStages;
-  uint64_t* done = empty + kStages;
+  uint64_t* full = reinterpret_cast<uint64_t*>(base + stages * kStageBytes);
+  uint64_t* empty = full + stages;
+  uint64_t* done = empty + stages;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * kBN;
   const int nkb0 = K / kBK, nkb = 3 * nkb0;  // three K-segments of the split product
-  float* s_lh = reinterpret_cast<float*>(base + kStages * kStageBytes + 256);
-  const int m = m0 + warp * 32 + lane;  // this thread's accumulator row in the epilogue
-  float lwm = 0.f;
-  uint32_t zbits[kBN / 32] = {};        // Epi 2: mask bits of this thread's 128 outputs
-  if (EPI == kEpiBf16TScale) {
-    s_lh[threadIdx.x] = o.lh[n0 + threadIdx.x];
-    lwm = o.lw[m];
-  } else if (EPI == kEpiF64TMask) {
-    // four coalesced words, issued before the main loop so they overlap the MMAs
-    if (o.mbits) {
-#pragma unroll
-      for (int w = 0; w < kBN / 32; ++w) zbits[w] = __ldg(o.mbits + (size_t)((n0 >> 5) + w) * o.ldb + m);
-    }
-  }
+  float* s_lh = reinterpret_cast<float*>(base + stages * kStageBytes + 256);
+  if (EPI == kEpiBf16TScale && threadIdx.x < kBN) s_lh[threadIdx.x] = o.lh[n0 + threadIdx.x];
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < stages; ++s) {
       mbar_init(full + s, 1);
       mbar_init(empty + s, 1);
     }
@@ -116,62 +112,89 @@ __global__ void __launch_bounds__(128, 1) k_gemm_nt(const __grid_constant__ CUte
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 4) {
     // TMA producer
-    for (int kb = 0; kb < nkb; ++kb) {
-      const int s = kb % kStages, u = kb / kStages;
-      if (u > 0 && !mbar_wait(empty + s, (u - 1) & 1, o.err)) break;
-      unsigned char* sa = base + s * kStageBytes;
-      const int seg = kb / nkb0, kc = (kb - seg * nkb0) * kBK;
-      mbar_expect_tx(full + s, kStageBytes);
-      tma_load_2d(sa, seg == 2 ? &tmAl : &tmA, full + s, kc, m0);
-      tma_load_2d(sa + kTileBytes, seg == 1 ? &tmBl : &tmB, full + s, kc, n0);
-    }
-  } else if (warp == 1 && lane == 0) {
-    // MMA issuer: four K = 16 steps per 64-wide stage, advancing the descriptors by 32 bytes
-    bool ok = true;
-    for (int kb = 0; kb < nkb && ok; ++kb) {
-      const int s = kb % kStages, u = kb / kStages;
-      if (!mbar_wait(full + s, u & 1, o.err)) {
-        ok = false;
-        break;
+    if (lane == 0) {
+      for (int kb = 0, s = 0, u = 0; kb < nkb; ++kb) {
+        if (u > 0 && !mbar_wait(empty + s, (u - 1) & 1, o.err)) break;
+        unsigned char* sa = base + s * kStageBytes;
+        const int seg = kb / nkb0, kc = (kb - seg * nkb0) * kBK;
+        mbar_expect_tx(full + s, kStageBytes);
+        tma_load_2d(sa, seg == 2 ? &tmAl : &tmA, full + s, kc, m0);
+        tma_load_2d(sa + kTileBytes, seg == 1 ? &tmBl : &tmB, full + s, kc, n0);
+        if (++s == stages) {
+          s = 0;
+          ++u;
+        }
       }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const unsigned char* sa = base + s * kStageBytes;
-      const uint64_t da = sw128_desc(sa), db = sw128_desc(sa + kTileBytes);
-#pragma unroll
-      for (int kk = 0; kk < kBK / 16; ++kk)
-        mma_bf16(tmem, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), kIdesc, (kb | kk) != 0);
-      mma_commit(empty + s);
     }
-    mma_commit(done);
-  }
-  __syncwarp();
-
-  // epilogue: warp w owns accumulator lanes (rows m) 32w .. 32w+31
-  const bool ready = __all_sync(0xffffffffu, mbar_wait(done, 0, o.err));
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (ready) {
-#pragma unroll 1
-    for (int c = 0; c < kBN / 16; ++c) {
-      float v[16];
-      tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * 16), v);
+    __syncwarp();
+  } else if (warp == 5) {
+    // MMA issuer: four K = 16 steps per 64-wide stage, advancing the descriptors by 32 bytes
+    if (lane == 0) {
+      for (int kb = 0, s = 0, u = 0; kb < nkb; ++kb) {
+        if (!mbar_wait(full + s, u & 1, o.err)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const unsigned char* sa = base + s * kStageBytes;
+        const uint64_t da = sw128_desc(sa), db = sw128_desc(sa + kTileBytes);
 #pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        const int n = n0 + c * 16 + q;
-        const size_t off = (size_t)n * o.ldo + m;
-        if (EPI == kEpiBf16T || EPI == kEpiBf16TScale) {
-          float w = v[q];
-          // 1/Lambda(a, b) with a = n, b = m; the zero mode and the padding give 0
-          if (EPI == kEpiBf16TScale) w *= (n | m) ? 1.f / (s_lh[c * 16 + q] + lwm) : 0.f;
-          const __nv_bfloat16 h = __float2bfloat16_rn(w);
-          reinterpret_cast<__nv_bfloat16*>(o.out)[off] = h;
-          reinterpret_cast<__nv_bfloat16*>(o.out_lo)[off] = __float2bfloat16_rn(w - __bfloat162float(h));
-        } else {
-          if (n < o.rows && m < o.cols) {
-            const int nn = c * 16 + q;
-            const bool z = (zbits[nn >> 5] >> (nn & 31)) & 1u;
-            reinterpret_cast<double*>(o.out)[off] = z ? 0.0 : (double)v[q];
+        for (int kk = 0; kk < kBK / 16; ++kk)
+          mma_bf16(tmem, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), kIdesc, (kb | kk) != 0);
+        mma_commit(empty + s);
+        if (++s == stages) {
+          s = 0;
+          ++u;
+        }
+      }
+      mma_commit(done);
+    }
+    __syncwarp();
+  } else {
+    // epilogue: warp w owns accumulator lanes (rows m) 32w .. 32w+31.  What it needs beside the
+    // accumulator is made while the main loop runs: the divisions of 1/Lambda after it (128 per
+    // thread) took 9 of the second product's 31 us at 1024x1024.
+    const int m = m0 + warp * 32 + lane;
+    uint32_t zbits[kBN / 32] = {};  // Epi 2: mask bits of this thread's 128 outputs
+    float inv[EPI == kEpiBf16TScale ? kBN : 1];
+    if (EPI == kEpiBf16TScale) {
+      const float lwm = o.lw[m];
+      // 1/Lambda(a, b) with a = n, b = m; the zero mode and the padding give 0
+#pragma unroll
+      for (int q = 0; q < kBN; ++q) inv[EPI == kEpiBf16TScale ? q : 0] = ((n0 + q) | m) ? 1.f / (s_lh[q] + lwm) : 0.f;
+    } else if (EPI == kEpiF64TMask) {
+      if (o.mbits) {
+#pragma unroll
+        for (int w = 0; w < kBN / 32; ++w) zbits[w] = __ldg(o.mbits + (size_t)((n0 >> 5) + w) * o.ldb + m);
+      }
+    }
+    const bool ready = __all_sync(0xffffffffu, mbar_wait(done, 0, o.err));
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (ready) {
+#pragma unroll
+      for (int c = 0; c < kBN / 16; ++c) {
+        float v[16];
+        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * 16), v);
+        bool plain = true;
+        if (EPI == kEpiF64TMask) {
+#pragma unroll
+          for (int q = 0; q < 16; ++q) plain &= is_plain(v[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+          const int n = n0 + c * 16 + q;
+          const size_t off = (size_t)n * o.ldo + m;
+          if (EPI == kEpiBf16T || EPI == kEpiBf16TScale) {
+            float w = v[q];
+            if (EPI == kEpiBf16TScale) w *= inv[EPI == kEpiBf16TScale ? c * 16 + q : 0];
+            const __nv_bfloat16 h = __float2bfloat16_rn(w);
+            reinterpret_cast<__nv_bfloat16*>(o.out)[off] = h;
+            reinterpret_cast<__nv_bfloat16*>(o.out_lo)[off] = __float2bfloat16_rn(w - __bfloat162float(h));
+          } else {
+            if (n < o.rows && m < o.cols) {
+              const int nn = c * 16 + q;
+              const bool z = (zbits[nn >> 5] >> (nn & 31)) & 1u;
+              reinterpret_cast<double*>(o.out)[off] = z ? 0.0 : plain ? widen_plain(v[q]) : widen(v[q]);
+            }
           }
         }
       }
@@ -213,13 +236,13 @@ __global__ void k_mask_bits(const uint8_t* __restrict__ mask, int H, int W, int 
 }
 
 // ------------------------------------------------------------------ host side
-// 2-D BF16 tensor [rows][cols] (cols contiguous), box 64 x 128, 128-byte swizzle.
-static bool make_map(CUtensorMap* tm, const void* ptr, int rows, int cols) {
+// 2-D BF16 tensor [rows][cols] (cols contiguous), box 64 x box_rows, 128-byte swizzle.
+static bool make_map(CUtensorMap* tm, const void* ptr, int rows, int cols, int box_rows) {
   PFN_encodeTiled fn = encode_fn();
   if (!fn) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-  const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)kBM};
+  const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -229,9 +252,13 @@ static bool make_map(CUtensorMap* tm, const void* ptr, int rows, int cols) {
 // dynamic shared memory above 48 KB is an attribute of the function on the current device:
 // set when a plan is made on it
 static void gemm_attrs() {
-  cudaFuncSetAttribute(k_gemm_nt<kEpiBf16T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
-  cudaFuncSetAttribute(k_gemm_nt<kEpiBf16TScale>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
-  cudaFuncSetAttribute(k_gemm_nt<kEpiF64TMask>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
+  auto set = [](auto* k) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(kRingBytes)); };
+  set(k_gemm_nt<kEpiBf16T, 64>);
+  set(k_gemm_nt<kEpiBf16T, 128>);
+  set(k_gemm_nt<kEpiBf16TScale, 64>);
+  set(k_gemm_nt<kEpiBf16TScale, 128>);
+  set(k_gemm_nt<kEpiF64TMask, 64>);
+  set(k_gemm_nt<kEpiF64TMask, 128>);
 }
 
 // A split operand: its high and low BF16 planes.
@@ -240,15 +267,21 @@ struct Split {
   const void* l;
 };
 
-template <int EPI>
-static cudaError_t gemm(Split A, int M, Split B, int N, int K, const GemmOut& o, cudaStream_t st) {
+template <int EPI, int BN>
+static cudaError_t gemm_bn(Split A, int M, Split B, int N, int K, const GemmOut& o, int nsm, cudaStream_t st) {
   CUtensorMap ta, tb, tal, tbl;
-  if (!make_map(&ta, A.h, M, K) || !make_map(&tb, B.h, N, K) || !make_map(&tal, A.l, M, K) ||
-      !make_map(&tbl, B.l, N, K))
+  if (!make_map(&ta, A.h, M, K, kBM) || !make_map(&tb, B.h, N, K, BN) || !make_map(&tal, A.l, M, K, kBM) ||
+      !make_map(&tbl, B.l, N, K, BN))
     return cudaErrorInvalidValue;
-  dim3 grid(N / kBN, M / kBM);
-  k_gemm_nt<EPI><<<grid, 128, kGemmSmem, st>>>(ta, tb, tal, tbl, K, o);
+  dim3 grid(N / BN, M / kBM);
+  const int stages = (int)(grid.x * grid.y) <= nsm ? kRingBytes / stage_bytes(BN) : kStagesMany;
+  k_gemm_nt<EPI, BN><<<grid, kGemmThreads, gemm_smem(stages * stage_bytes(BN)), st>>>(ta, tb, tal, tbl, K, stages, o);
   return cudaGetLastError();
+}
+template <int EPI>
+static cudaError_t gemm(Split A, int M, Split B, int N, int K, const GemmOut& o, int nsm, cudaStream_t st) {
+  if ((long long)(M / kBM) * (N / 128) * 2 <= nsm) return gemm_bn<EPI, 64>(A, M, B, N, K, o, nsm, st);
+  return gemm_bn<EPI, 128>(A, M, B, N, K, o, nsm, st);
 }
 
 // Orthonormal DCT-II matrix of size n padded to np, C[k][x] = c_k cos(pi k (x + 1/2) / n),
@@ -274,6 +307,7 @@ static void dct_matrix(int n, int np, std::vector<__nv_bfloat16>& C, std::vector
 // Device buffers of the DCT preconditioner for an H x W map (allocated with the plan).
 struct DctPlan {
   int H = 0, W = 0, Hp = 0, Wp = 0;
+  int nsm = 1;
   __nv_bfloat16 *CH = nullptr, *CHT = nullptr, *CW = nullptr, *CWT = nullptr;      // high planes
   __nv_bfloat16 *CHl = nullptr, *CHTl = nullptr, *CWl = nullptr, *CWTl = nullptr;  // low planes
   __nv_bfloat16 *R = nullptr, *X = nullptr, *Y = nullptr;     // R, X^T / S^, Y^T (high)
@@ -343,9 +377,10 @@ int dct_setup(DctPlan& d, int H, int W, void* mem) {
   return 0;
 }
 
-DctPlan* dct_create(int H, int W, void* mem) {
+DctPlan* dct_create(int H, int W, void* mem, int nsm) {
   gemm_attrs();
   DctPlan* d = new DctPlan();
+  d->nsm = nsm;
   if (dct_setup(*d, H, W, mem) != 0) {
     delete d;
     return nullptr;
@@ -391,7 +426,7 @@ cudaError_t dct_apply(const DctPlan& d, const double* r, int pitch, const uint8_
   o.out = d.X;
   o.out_lo = d.Xl;
   o.ldo = Hp;
-  cudaError_t e = gemm<kEpiBf16T>({d.R, d.Rl}, Hp, {d.CW, d.CWl}, Wp, Wp, o, st);
+  cudaError_t e = gemm<kEpiBf16T>({d.R, d.Rl}, Hp, {d.CW, d.CWl}, Wp, Wp, o, d.nsm, st);
   if (e != cudaSuccess) return e;
   // G2: S^[a][b] = (sum_i X^T[b][i] C_H[a][i]) / Lambda[a][b]
   o.out = d.Y;
@@ -399,14 +434,14 @@ cudaError_t dct_apply(const DctPlan& d, const double* r, int pitch, const uint8_
   o.ldo = Wp;
   o.lh = d.lh;
   o.lw = d.lw;
-  e = gemm<kEpiBf16TScale>({d.X, d.Xl}, Wp, {d.CH, d.CHl}, Hp, Hp, o, st);
+  e = gemm<kEpiBf16TScale>({d.X, d.Xl}, Wp, {d.CH, d.CHl}, Hp, Hp, o, d.nsm, st);
   if (e != cudaSuccess) return e;
   // G3: Y^T[j][a] = sum_b S^[a][b] C_W^T[j][b]
   o.out = d.X;
   o.out_lo = d.Xl;
   o.ldo = Hp;
   o.lh = o.lw = nullptr;
-  e = gemm<kEpiBf16T>({d.Y, d.Yl}, Hp, {d.CWT, d.CWTl}, Wp, Wp, o, st);
+  e = gemm<kEpiBf16T>({d.Y, d.Yl}, Hp, {d.CWT, d.CWTl}, Wp, Wp, o, d.nsm, st);
   if (e != cudaSuccess) return e;
   // G4: S[i][j] = sum_a Y^T[j][a] C_H^T[i][a], masked, into the FP64 plane
   o.out = s;
@@ -416,7 +451,7 @@ cudaError_t dct_apply(const DctPlan& d, const double* r, int pitch, const uint8_
   o.ldb = Wp;
   o.rows = d.H;
   o.cols = d.W;
-  return gemm<kEpiF64TMask>({d.X, d.Xl}, Wp, {d.CHT, d.CHTl}, Hp, Hp, o, st);
+  return gemm<kEpiF64TMask>({d.X, d.Xl}, Wp, {d.CHT, d.CHTl}, Hp, Hp, o, d.nsm, st);
 }
 
 }  // namespace ulp

@@ -104,7 +104,7 @@ void launch_pcg_reset(const Plan& pl, cudaStream_t st, bool flow = false);
 
 // ulp_dct.cu
 size_t dct_bytes(int H, int W);
-DctPlan* dct_create(int H, int W, void* mem);  // builds the matrices in mem (dct_bytes); null on failure
+DctPlan* dct_create(int H, int W, void* mem, int nsm);  // builds the matrices in mem (dct_bytes); null on failure
 void dct_destroy(DctPlan* d);
 // the split BF16 copy of r that the first GEMM reads: high plane returned, low plane in *lo
 unsigned* dct_input(const DctPlan& d, int* ld_pairs, unsigned** lo);
