@@ -206,11 +206,16 @@ static int plan_init(Plan& pl, int n, const int* H, const int* W, const ulp_opti
   // on small maps are more than the tiles (in FP64 the dot phase rides there only where they
   // are not)
   constexpr int kMgUnits = 2048;
-  const int npart = tiles > kMgUnits ? tiles : kMgUnits;
+  int npart = tiles > kMgUnits ? tiles : kMgUnits;
+  if (n == 1) {  // the mixed flexible CG's own tiles
+    const MapDesc& M = pl.hmaps[0];
+    const int R = fcg_mixed_rows(M.H, M.nsx, pl.nsm), nt = M.nsx * ((M.H + R - 1) / R);
+    if (nt > npart) npart = nt;
+  }
   const size_t off_part = bytes;
   bytes += 3 * align256(sizeof(double) * npart);
   const size_t off_flow = bytes;
-  pl.nflow = tiles > pl.nsm + n ? tiles : pl.nsm + n;
+  pl.nflow = npart > pl.nsm + n ? npart : pl.nsm + n;
   bytes += align256(sizeof(double) * kFlowSlots * pl.nflow);
   const size_t off_outer = bytes;
   bytes += align256(sizeof(double) * 2 * (size_t)n * pl.bx_elem);
@@ -278,7 +283,8 @@ static int plan_init(Plan& pl, int n, const int* H, const int* W, const ulp_opti
       return fail(ULP_ERR_NOMEM, "cudaMalloc(multigrid levels): %s", cudaGetErrorString(e));
     }
     pl.mg = mg_create(pl.hmaps[0], pl.mg_mem, pl.nsm, pl.ntiles,
-                      pl.opt.precision == ULP_PRECISION_MIXED ? npart : pl.ntiles);
+                      pl.opt.precision == ULP_PRECISION_MIXED ? npart : pl.ntiles,
+                      pl.opt.precision == ULP_PRECISION_MIXED);
   }
   ULP_CU(cudaDeviceSynchronize());  // workspace zeroed before any stream may use it
   return ULP_OK;

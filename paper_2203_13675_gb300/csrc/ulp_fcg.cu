@@ -420,7 +420,7 @@ __device__ __forceinline__ XState x_state(const MapDesc& M, MapState* S) {
 }
 
 // One tile per warp.
-__global__ void __launch_bounds__(kThreads, 2) k_x_a(const __grid_constant__ FcgArgs f) {
+__global__ void __launch_bounds__(kThreads, 3) k_x_a(const __grid_constant__ FcgArgs f) {
   __shared__ Slot32 ring[kWarps][kRing32];  // the stencil's row rings
   const PcgArgs& a = f.a;
   const int lane = threadIdx.x & 31;
@@ -445,7 +445,7 @@ struct SlotB {
 constexpr size_t kRingBSmem = (size_t)kWarps * kRingB * sizeof(SlotB);  // 71,680 bytes
 
 // alpha, then the phase's updates.  One tile per warp.
-__global__ void __launch_bounds__(kThreads, 2) k_x_b(const __grid_constant__ FcgArgs f) {
+__global__ void __launch_bounds__(kThreads, 3) k_x_b(const __grid_constant__ FcgArgs f) {
   extern __shared__ __align__(16) unsigned char xb_dsm[];
   const PcgArgs& a = f.a;
   const int lane = threadIdx.x & 31;
@@ -657,7 +657,7 @@ __global__ void __launch_bounds__(kThreads) k_f_jacobi(const __grid_constant__ F
   }
 }
 
-static int tile_blocks(const Plan& pl) { return (pl.ntiles + kWarps - 1) / kWarps; }
+static int tile_blocks(const FcgArgs& f) { return (f.a.ntiles + kWarps - 1) / kWarps; }
 
 // s = M^-1 r of the flexible solve: the DCT chain, or the network followed by its
 // Jacobi fallback (only one of the two does work in any iteration).
@@ -679,7 +679,7 @@ static cudaError_t fcg_precond(Plan& pl, int kind, const FcgArgs& f, cudaStream_
   const cudaError_t e = unet_apply_plane(*pl.unet, M.f.r, M.f.U, M.f.V, M.f.mask, M.H, M.W, M.pitch, M.f.s,
                                          &pl.dstate[0].fallback, st);
   if (e != cudaSuccess) return e;
-  k_f_jacobi<<<tile_blocks(pl), kThreads, 0, st>>>(f);
+  k_f_jacobi<<<tile_blocks(f), kThreads, 0, st>>>(f);
   return cudaGetLastError();
 }
 
@@ -689,7 +689,7 @@ static bool fused_dots(const Plan& pl, int kind) { return kind == ULP_PRECOND_MG
 // The scalars after the start (init) or a body's dot phase.
 static void fcg_finish(Plan& pl, int kind, const FcgArgs& f, bool fd, bool init, cudaStream_t st) {
   const bool x = mixed_fcg(pl, kind);
-  const int nb = tile_blocks(pl), nt = pl.ntiles, nu = fd ? mg_dot_units(*pl.mg) : nt;
+  const int nb = tile_blocks(f), nt = f.a.ntiles, nu = fd ? mg_dot_units(*pl.mg) : nt;
   // r^T r comes from the dot phase's kernel, but in the fused mixed form from those that wrote
   // r; the third sum from phase B, the residual, or k_f_dots / k_x_dots at the start
   const bool b1 = x && fd, b2 = x && (fd || !init);
@@ -700,7 +700,7 @@ static void fcg_finish(Plan& pl, int kind, const FcgArgs& f, bool fd, bool init,
 // Start of a solve: r = b - A phi (and its BF16 copy), the mask bits, s = M^-1 r, delta_0.
 static cudaError_t fcg_start(Plan& pl, int kind, const FcgArgs& f, cudaStream_t st) {
   const MapDesc& M = pl.hmaps[0];
-  const int nb = tile_blocks(pl);
+  const int nb = tile_blocks(f);
   const bool stamp = pl.opt.profile != 0;
   if (mixed_fcg(pl, kind)) {
     const bool fd = fused_dots(pl, kind);
@@ -729,7 +729,7 @@ static cudaError_t fcg_start(Plan& pl, int kind, const FcgArgs& f, cudaStream_t 
 
 // One iteration: A, B, R, s = M^-1 r, D.
 static cudaError_t fcg_iteration(Plan& pl, int kind, const FcgArgs& f, cudaStream_t st) {
-  const int nb = tile_blocks(pl);
+  const int nb = tile_blocks(f);
   const bool fd = fused_dots(pl, kind);
   if (mixed_fcg(pl, kind)) {
     k_x_a<<<nb, kThreads, 0, st>>>(f);
@@ -796,7 +796,7 @@ static cudaError_t fcg_build(Plan& pl, int kind, FcgArgs f) {
   }
   if (e == cudaSuccess) e = cudaStreamUpdateCaptureDependencies(st, &cn, nullptr, 1, cudaStreamSetCaptureDependencies);
   if (e == cudaSuccess && mixed_fcg(pl, kind)) {
-    k_x_fold<<<tile_blocks(pl), kThreads, 0, st>>>(f);
+    k_x_fold<<<tile_blocks(f), kThreads, 0, st>>>(f);
     e = cudaGetLastError();
   }
   cudaGraph_t gout = nullptr;
@@ -835,7 +835,7 @@ static cudaError_t fcg_build(Plan& pl, int kind, FcgArgs f) {
 // host launch, so a profiler sees each one; the host reads the stop flag after
 // every iteration.  For measurement only.
 static cudaError_t fcg_eager_mixed(Plan& pl, int kind, const FcgArgs& f, cudaStream_t st) {
-  const int nb = tile_blocks(pl);
+  const int nb = tile_blocks(f);
   const bool fd = fused_dots(pl, kind);
   cudaError_t e = fcg_attrs();
   if (e != cudaSuccess) return e;
@@ -875,7 +875,7 @@ static cudaError_t fcg_eager_mixed(Plan& pl, int kind, const FcgArgs& f, cudaStr
 static cudaError_t fcg_eager(Plan& pl, int kind, const FcgArgs& f, cudaStream_t st) {
   if (mixed_fcg(pl, kind)) return fcg_eager_mixed(pl, kind, f, st);
   const MapDesc& M = pl.hmaps[0];
-  const int nb = tile_blocks(pl);
+  const int nb = tile_blocks(f);
   cudaError_t e = fcg_attrs();
   if (e != cudaSuccess) return e;
   phase_mark(pl, st, -1);
@@ -919,6 +919,30 @@ static cudaError_t fcg_eager(Plan& pl, int kind, const FcgArgs& f, cudaStream_t 
   return cudaGetLastError();
 }
 
+// Tiles of the solve: the plan's, one wave of two blocks per SM, up to the size where the
+// plan's tiles reach their 64 rows and become more than a wave.  Beyond it the mixed form,
+// whose sums are per block, takes one wave of three blocks per SM (k_x_a and k_x_b are built
+// for that): at 4096x4096 72 rows, 456 blocks, k_x_a 102 -> 82 us and k_x_b 86 -> 83 (the
+// plan's 4096 tiles are 512 blocks).  At 2048x2048 three blocks per SM, 18 rows instead of
+// 27, measured slower (k_x_a 23.9 us against 22.7).
+constexpr int kXBlocksPerSm = 3;
+int fcg_mixed_rows(int H, int nsx, int nsm) {
+  const long long warps = (long long)nsm * kXBlocksPerSm * kWarps;
+  long long R = ((long long)H * nsx + warps - 1) / warps;
+  if (R < 4) R = 4;
+  while (R < H && (long long)nsx * ((H + R - 1) / R) > warps) ++R;  // a ragged last band counts too
+  return (int)R;
+}
+static FcgArgs fcg_args(const Plan& pl, const PcgArgs& a) {
+  FcgArgs f{a, pl.hmaps[0], pl.dargs};
+  if (a.xfcg && pl.ntiles > 2 * kWarps * pl.nsm) {
+    f.a.R = fcg_mixed_rows(f.M.H, f.M.nsx, pl.nsm);
+    f.M.nsy = (f.M.H + f.a.R - 1) / f.a.R;
+    f.a.ntiles = f.M.ntiles = f.M.nsx * f.M.nsy;
+  }
+  return f;
+}
+
 cudaError_t launch_fcg(Plan& pl, int kind, const PcgArgs& a_in, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1) {
   if (pl.nmaps != 1) return cudaErrorNotSupported;
   if (kind == ULP_PRECOND_DCT && !pl.dct) return cudaErrorNotSupported;
@@ -939,7 +963,7 @@ cudaError_t launch_fcg(Plan& pl, int kind, const PcgArgs& a_in, cudaStream_t st,
   if (kind == ULP_PRECOND_MG && !a.xfcg) a.rf32 = mg_input(*pl.mg);
   a.learned = kind == ULP_PRECOND_LEARNED;
   a.cond = 0;
-  const FcgArgs f{a, pl.hmaps[0], pl.dargs};
+  const FcgArgs f = fcg_args(pl, a);
   if (pl.opt.profile == 2) {
     k_set_args<<<1, 1, 0, st>>>(a, pl.dargs);
     launch_pcg_reset(pl, st);

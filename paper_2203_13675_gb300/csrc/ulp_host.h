@@ -120,7 +120,7 @@ int dct_error(const DctPlan& d);  // 1 if a GEMM wait ran out since the last cal
 // ulp_mg.cu: aggregation multigrid on the map's planes (U, V, D^-1; r -> s, y as scratch)
 size_t mg_bytes(int H, int W);
 // max_units: partials of the map grid's last kernel that the plan has room for
-MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles, int max_units);
+MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles, int max_units, bool mixed);
 void mg_destroy(MgPlan* p);
 // coarse grids, once per solve; level0: make the map grid's FP32 weights and D^-1 from the FP64
 // planes (false when launch_system_x already wrote them)
@@ -166,6 +166,7 @@ int matvec_on_plan(ulp_plan plan, const double* U, const double* V, const double
 cudaError_t launch_fcg(Plan& pl, int kind, const PcgArgs& a, cudaStream_t st, cudaEvent_t e0 = nullptr,
                        cudaEvent_t e1 = nullptr);
 void destroy_fcg(Plan& pl);
+int fcg_mixed_rows(int H, int nsx, int nsm);  // rows per tile of the mixed flexible CG
 
 // ulp_resident.cu: the Jacobi / identity solvers with their working set on the chip; whether
 // the plan's tiles fit, and the launch (attributes are set on the current device first)

@@ -807,16 +807,27 @@ __global__ void __launch_bounds__(kWalkWarps * 32) k_mg_down_w(Grid f, Grid c, i
 }
 
 // one slot of the up walker's ring: U, V, D^-1, b, x of row r, the coarse x of its
-// aggregates, and on the map's grid the mask and FP64 r of row r - 2
-struct UpSlot {
+// aggregates, and on the map's grid the mask and, in the FP64 form, r of row r - 2.  Without
+// that r a block's ring is 47 KB instead of 63 and four blocks fit an SM instead of three.
+struct UpSlotBase {
   float4 U[32], V[32], D[32], B[32], X[32];
   float2 XC[32];
   uchar4 MK[32];
+};
+struct UpSlot64 : UpSlotBase {
   double2 RA[32], RB[32];
+};
+template <int MODE>
+struct UpSlotOf {
+  using T = UpSlotBase;
+};
+template <>
+struct UpSlotOf<kUp64> {
+  using T = UpSlot64;
 };
 
 template <int MODE>
-__device__ __forceinline__ void up_issue(UpSlot& sl, const Grid& f, const Grid& c, const float* xc,
+__device__ __forceinline__ void up_issue(typename UpSlotOf<MODE>::T& sl, const Grid& f, const Grid& c, const float* xc,
                                          const uint8_t* mask, const double* rv, int r, int j, int lane) {
   const int nb = row_bytes(f, r, j);
   const size_t o = nb ? (size_t)r * f.ld + j : 0;
@@ -831,9 +842,11 @@ __device__ __forceinline__ void up_issue(UpSlot& sl, const Grid& f, const Grid& 
     const int pb = row_bytes(f, p, j);
     const size_t op = pb ? (size_t)p * f.ld + j : 0;
     if (mask) cp_async4(&sl.MK[lane], mask + op, pb ? 4 : 0);
-    if (MODE == kUp64 && rv) {
-      cp_async16(&sl.RA[lane], rv + op, pb ? 16 : 0);
-      cp_async16(&sl.RB[lane], rv + op + (pb ? 2 : 0), pb ? 16 : 0);
+    if constexpr (MODE == kUp64) {
+      if (rv) {
+        cp_async16(&sl.RA[lane], rv + op, pb ? 16 : 0);
+        cp_async16(&sl.RB[lane], rv + op + (pb ? 2 : 0), pb ? 16 : 0);
+      }
     }
   }
 }
@@ -851,6 +864,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32) k_mg_up_w(Grid f, Grid c, con
   int seg, band, j, lane;
   const int bands = (f.H + R - 1) / R;
   if (!walk_warp(f.W, bands, seg, band, j, lane)) return;
+  using UpSlot = typename UpSlotOf<MODE>::T;
   UpSlot* ring = reinterpret_cast<UpSlot*>(wsm4) + (threadIdx.x >> 5) * kRing;
   const bool out = lane >= 1 && lane <= 30 && j < f.W;
   const int i0 = band * R, i1 = min(f.H, i0 + R);
@@ -915,15 +929,17 @@ __global__ void __launch_bounds__(kWalkWarps * 32) k_mg_up_w(Grid f, Grid c, con
             for (int k = 0; k < 4; ++k)
               if (j + k < f.W) s[o + k] = sv[k];
           }
-          if (rv) {
-            const double2 ra = sl.RA[lane], rb2 = sl.RB[lane];
-            const double rk[4] = {ra.x, ra.y, rb2.x, rb2.y};
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-              if (j + k < f.W) {
-                rs = fma(rk[k], sv[k], rs);
-                rr = fma(rk[k], rk[k], rr);
-              }
+          if constexpr (MODE == kUp64) {
+            if (rv) {
+              const double2 ra = sl.RA[lane], rb2 = sl.RB[lane];
+              const double rk[4] = {ra.x, ra.y, rb2.x, rb2.y};
+  #pragma unroll
+              for (int k = 0; k < 4; ++k)
+                if (j + k < f.W) {
+                  rs = fma(rk[k], sv[k], rs);
+                  rr = fma(rk[k], rk[k], rr);
+                }
+          }
           }
         }
       }
@@ -943,7 +959,8 @@ __global__ void __launch_bounds__(kWalkWarps * 32) k_mg_up_w(Grid f, Grid c, con
 }
 
 constexpr size_t kDownRingSmem = (size_t)kWalkWarps * kRing * sizeof(DownSlot);
-constexpr size_t kUpRingSmem = (size_t)kWalkWarps * kRing * sizeof(UpSlot);
+template <int MODE>
+constexpr size_t kUpRingSmem = (size_t)kWalkWarps * kRing * sizeof(typename UpSlotOf<MODE>::T);
 
 // level 0 without the fused kernels (grids narrower than 64 columns): the FP64 s rounded to FP32
 __global__ void k_mg_to32(const double* __restrict__ s, float* s32, Grid g, const MapState* S) {
@@ -1240,7 +1257,7 @@ static unsigned tile_blocks(const Grid& f, int TR) {
   return (unsigned)(((f.W + kSegOut - 1) / kSegOut) * ((f.H + TR - 1) / TR));
 }
 
-MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles, int max_units) {
+MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles, int max_units, bool mixed) {
   MgPlan* p = new MgPlan();
   p->mem = mem;
   p->nsm = nsm;
@@ -1296,17 +1313,25 @@ MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles, int max_unit
     cudaFuncSetAttribute(k_mg_up_t<kUp64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem);
     cudaFuncSetAttribute(k_mg_up_t<kUp32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem);
     cudaFuncSetAttribute(k_mg_down_w, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDownRingSmem);
-    cudaFuncSetAttribute(k_mg_up_w<kUpCoarse>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpRingSmem);
-    cudaFuncSetAttribute(k_mg_up_w<kUp64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpRingSmem);
-    cudaFuncSetAttribute(k_mg_up_w<kUp32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpRingSmem);
+    cudaFuncSetAttribute(k_mg_up_w<kUpCoarse>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpRingSmem<kUpCoarse>);
+    cudaFuncSetAttribute(k_mg_up_w<kUp64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpRingSmem<kUp64>);
+    cudaFuncSetAttribute(k_mg_up_w<kUp32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpRingSmem<kUp32>);
   }
-  // one resident wave of each walker (the ring's shared memory limits the up walker to
-  // three blocks per SM): more warps than that run as a second, mostly idle wave
-  int occ_down = 0, occ_up = 0;
+  // one resident wave of each walker: more warps than that run as a second, mostly idle wave.
+  // The mixed form's map grid takes the four blocks per SM that its smaller ring allows where
+  // that leaves bands of kTallBand rows at least (a band reads four rows of halo): at
+  // 4096x4096 59 rows instead of 79, 87 -> 81 us; at 2048x2048 16 rows instead of 21 measured
+  // 26.3 us against 25.6.
+  int occ_down = 0, occ_up = 0, occ_up32 = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_down, k_mg_down_w, kWalkWarps * 32, kDownRingSmem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_up, k_mg_up_w<kUp32>, kWalkWarps * 32, kUpRingSmem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_up, k_mg_up_w<kUp64>, kWalkWarps * 32, kUpRingSmem<kUp64>);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_up32, k_mg_up_w<kUp32>, kWalkWarps * 32, kUpRingSmem<kUp32>);
   const long long wave_down = (long long)(occ_down > 0 ? occ_down : 1) * kWalkWarps * nsm;
   const long long wave_up = (long long)(occ_up > 0 ? occ_up : 1) * kWalkWarps * nsm;
+  const long long wave_up32 = (long long)(occ_up32 > 0 ? occ_up32 : 1) * kWalkWarps * nsm;
+  constexpr int kTallBand = 32;
+  long long wave_map = wave_up < ntiles ? wave_up : ntiles;
+  if (mixed && wave_up32 <= max_units && walk_rows(M.H, M.W, 2, wave_up32) >= kTallBand) wave_map = wave_up32;
   // walkers where even two-row bands fill a wave, tiles on the smaller grids (see the
   // walker section for the measurements)
   const long long wave = wave_up < wave_down ? wave_up : wave_down;
@@ -1318,7 +1343,7 @@ MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles, int max_unit
       if (nseg * ((f.H + 1) / 2) >= wave) {
         kind = kWalk;
         rd = walk_rows(p->g[l + 1].H, f.W, 1, wave_down);
-        ru = walk_rows(f.H, f.W, 2, l == 0 ? (wave_up < ntiles ? wave_up : ntiles) : wave_up);
+        ru = walk_rows(f.H, f.W, 2, l == 0 ? wave_map : wave_up);
       } else {
         kind = kTile;
         rd = tile_rows(f.H, f.W, nsm, true);
@@ -1333,8 +1358,8 @@ MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles, int max_unit
     const long long n = p->kind[0] == kWalk
                             ? (long long)((M.W + kSegOut - 1) / kSegOut) * ((M.H + p->rows_up[0] - 1) / p->rows_up[0])
                             : (long long)tile_blocks(p->g[0], p->rows_up[0]);
-    // (FP64 plans, max_units = ntiles: not on the smallest maps, whose sums keep the tiles' order)
-    if (n <= max_units && (n >= kArriveGroups || max_units > ntiles)) p->dots_units = (int)n;
+    // (FP64: not on the smallest maps, whose sums keep the tiles' order)
+    if (n <= max_units && (n >= kArriveGroups || mixed)) p->dots_units = (int)n;
   }
 
   // the tail: the smallest suffix of grids, from the first with at most kTailMax unknowns,
@@ -1421,9 +1446,9 @@ static void up_level(const MgPlan& p, int l, int stop, const uint8_t* mask, cons
     if (p.kind[l] == kWalk) {
       const unsigned nb = walk_blocks(f, f.H, R);
       const unsigned nt = kWalkWarps * 32;
-      if (mode == kUp32) k_mg_up_w<kUp32><<<nb, nt, kUpRingSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
-      else if (mode == kUp64) k_mg_up_w<kUp64><<<nb, nt, kUpRingSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
-      else k_mg_up_w<kUpCoarse><<<nb, nt, kUpRingSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
+      if (mode == kUp32) k_mg_up_w<kUp32><<<nb, nt, kUpRingSmem<kUp32>, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
+      else if (mode == kUp64) k_mg_up_w<kUp64><<<nb, nt, kUpRingSmem<kUp64>, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
+      else k_mg_up_w<kUpCoarse><<<nb, nt, kUpRingSmem<kUpCoarse>, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
     } else {
       const unsigned nb = tile_blocks(f, R);
       if (mode == kUp32) k_mg_up_t<kUp32><<<nb, kTileThreads, kTileSmem, st>>>(f, c, xc, R, mk, s64, rv, o32, d ? dots->P0 : nullptr, d ? dots->P1 : nullptr, S);
