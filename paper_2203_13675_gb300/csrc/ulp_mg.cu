@@ -202,15 +202,6 @@ __global__ void k_mg_level0(const double* __restrict__ U, const double* __restri
   }
 }
 
-// level 0: b = (float) r
-__global__ void k_mg_rhs(const double* __restrict__ r, Grid g, const MapState* S) {
-  if (skip_map(S)) return;
-  MG_LOOP(t, (long long)g.H * g.W) {
-    const size_t o = (size_t)(t / g.W) * g.ld + (t % g.W);
-    g.b[o] = (float)r[o];
-  }
-}
-
 // coarsest grid: thirty sweeps from zero in one block (x and t ping-pong)
 __global__ void k_mg_coarsest(Grid g, const MapState* S) {
   if (skip_map(S)) return;
