@@ -53,7 +53,10 @@ constexpr int stage_bytes(int BN) { return kTileBytes + BN * kBK * 2; }  // A + 
 // each, one's epilogue under the other's main loop.  The four products at 1024x1024 took
 // 22, 31, 22 and 26 us with 128 x 128 tiles, three stages and the epilogue's divisions at the
 // end, 19, 24, 19 and 27 with six stages and the divisions under way before, 18, 20, 18 and 22
-// as now (a DCT solve's call 29.5 -> 24.7 ms).
+// as now (a DCT solve's call 29.5 -> 24.7 ms).  The 128-wide builds are held to the registers
+// of two blocks: without that one of them takes 178, one block fits an SM, and where there are
+// more tiles than SMs a solve is slower than with 128 threads and three stages throughout
+// (2048x2048: 39.6 ms without, 35.1 with, 35.6 the older kernel; 1900x1300: 29.9, 25.8, 27.2).
 constexpr int kRingBytes = 6 * stage_bytes(kBNMax);  // 192 KB: six stages at BN = 128, eight at 64
 constexpr int kStagesMany = 3;
 constexpr int kGemmThreads = 192;  // warps 0-3 epilogue, warp 4 TMA, warp 5 MMA
@@ -76,7 +79,7 @@ struct GemmOut {
 // tmA / tmB: the high planes, tmAl / tmBl: the low planes; K-segments (Ah, Bh), (Ah, Bl),
 // (Al, Bh) in that order, all accumulated into one tensor-memory tile
 template <int EPI, int kBN>
-__global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_nt(const __grid_constant__ CUtensorMap tmA,
+__global__ void __launch_bounds__(kGemmThreads, kBN == kBNMax ? 2 : 1) k_gemm_nt(const __grid_constant__ CUtensorMap tmA,
                                                     const __grid_constant__ CUtensorMap tmB,
                                                     const __grid_constant__ CUtensorMap tmAl,
                                                     const __grid_constant__ CUtensorMap tmBl, int K, int stages,
