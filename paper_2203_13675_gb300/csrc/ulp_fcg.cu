@@ -844,10 +844,12 @@ static cudaError_t fcg_eager_mixed(Plan& pl, int kind, const FcgArgs& f, cudaStr
   phase_mark(pl, st, 2);
   if ((e = mg_setup(*pl.mg, pl.dstate, st, !pl.system_x)) != cudaSuccess) return e;
   if ((e = fcg_precond(pl, kind, f, st, fd)) != cudaSuccess) return e;
-  phase_mark(pl, st, 3);
-  if (!fd) k_x_dots<<<nb, kThreads, 0, st>>>(f, 1);
+  if (!fd) {
+    phase_mark(pl, st, 3);
+    k_x_dots<<<nb, kThreads, 0, st>>>(f, 1);
+  }
   fcg_finish(pl, kind, f, fd, true, st);
-  phase_mark(pl, st, 4);
+  phase_mark(pl, st, fd ? 3 : 4);
   for (long long l = 0;; ++l) {
     int done = 0;
     if ((e = cudaMemcpyAsync(&done, &pl.dstate->done, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
@@ -863,10 +865,12 @@ static cudaError_t fcg_eager_mixed(Plan& pl, int kind, const FcgArgs& f, cudaStr
     if ((e = fcg_precond(pl, kind, f, st, fd, 1)) != cudaSuccess) return e;
     phase_mark(pl, st, 3);
     if ((e = fcg_precond(pl, kind, f, st, fd, 2)) != cudaSuccess) return e;
-    phase_mark(pl, st, 5);
-    if (!fd) k_x_dots<<<nb, kThreads, 0, st>>>(f, 0);
+    if (!fd) {
+      phase_mark(pl, st, 5);
+      k_x_dots<<<nb, kThreads, 0, st>>>(f, 0);
+    }
     fcg_finish(pl, kind, f, fd, false, st);
-    phase_mark(pl, st, 4);
+    phase_mark(pl, st, fd ? 5 : 4);  // the closing sum counts to the phase that made the partials
   }
   k_x_fold<<<nb, kThreads, 0, st>>>(f);
   return cudaGetLastError();
@@ -907,14 +911,14 @@ static cudaError_t fcg_eager(Plan& pl, int kind, const FcgArgs& f, cudaStream_t 
       if ((e = fcg_precond(pl, kind, f, st, fd, 1)) != cudaSuccess) return e;
       phase_mark(pl, st, 3);
       if ((e = fcg_precond(pl, kind, f, st, fd, 2)) != cudaSuccess) return e;
-      phase_mark(pl, st, 5);
+      if (!fd) phase_mark(pl, st, 5);
     } else {
       if ((e = fcg_precond(pl, kind, f, st, fd)) != cudaSuccess) return e;
       phase_mark(pl, st, 3);
     }
     if (!fd) k_f_dots<<<nb, kThreads, 0, st>>>(f, 0);
     fcg_finish(pl, kind, f, fd, false, st);
-    phase_mark(pl, st, 4);
+    phase_mark(pl, st, fd ? 5 : 4);
   }
   return cudaGetLastError();
 }
