@@ -31,10 +31,9 @@
 
 #include "ulp_flow32.cuh"
 #include "ulp_host.h"
+#include "ulp_parts.h"
 
 namespace ulp {
-
-constexpr int kResMaxWarps = 16;
 
 template <typename T>
 struct Vec2;
@@ -337,7 +336,7 @@ struct ResShared {
   ResMap loc[kResMaxWarps];             // a block's tiles lie in at most that many maps
   MapDesc map[kResMaxWarps];
   double red[3][kResMaxWarps][32];      // lane sums of each warp's tile
-  double part[2][3][4];                 // by parity of the map's place, so that no round waits for the last one's reader
+  double part[kPartSlots][4];           // each map's and sum's own slot (ulp_parts.h)
   double sum[3];
   int n, alive, fail;
 };
@@ -373,7 +372,7 @@ __device__ __forceinline__ void res_begin(const PcgArgs& a, ResShared& sh, int p
   __syncthreads();
 }
 
-// The block's sum of one quantity over its tiles of a map (128 threads, r = 0 .. 127: warp k
+// The block's sum q over its tiles of the map at place i (128 threads, r = 0 .. 127: warp k
 // adds tiles k, k + 4, ... lane by lane and its lanes as a tree), published.
 __device__ __forceinline__ void res_publish(const PcgArgs& a, ResShared& sh, const ResMap& L, int i, int q, int r,
                                             double* slots, double* clear) {
@@ -381,7 +380,7 @@ __device__ __forceinline__ void res_publish(const PcgArgs& a, ResShared& sh, con
   double s = 0.0;
   for (int w = L.w0 + k; w < L.w1; w += 4) s += sh.red[q][w][lane];
   s = warp_sum(s);
-  double* p = sh.part[i & 1][q];
+  double* p = sh.part[part_slot(i, q)];
   if (lane == 0) p[k] = s;
   asm volatile("bar.sync %0, 128;" ::"r"((q & 1) + 1) : "memory");
   if (r == 0) {
