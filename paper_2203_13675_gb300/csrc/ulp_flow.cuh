@@ -240,8 +240,9 @@ __device__ __forceinline__ bool flow_step(const PcgArgs& a, FlowShared& fs) {
         }
       }
     }
+    // the verdict has been read by every thread before a wait for the next map may change it
+    __syncthreads();
   }
-  __syncthreads();
   return true;
 }
 
