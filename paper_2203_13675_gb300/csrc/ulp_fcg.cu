@@ -117,6 +117,36 @@ __device__ __forceinline__ void put_block_parts(const double (&v)[N], double* co
   }
 }
 
+// Solves of many tiles (many_tiles below): the group sums of three arrays of tile partials
+// (blockIdx.y: which, of n0 .. n2 partials) into the map's gpart, in tile_arrive's order.
+// Thread (l, g) of a block's four groups adds partials g + 32 (l + 32 k) in turn, then the
+// groups' lanes add up as tile_arrive's tree.  Eight blocks to an array: an SM adds 32 FP64
+// values in 64 cycles a partition, so one block took 8 us for 32768 tiles.
+constexpr int kGroupBlocks = 8;
+__global__ void __launch_bounds__(kSumThreads) k_f_groups(const __grid_constant__ FcgArgs f, int n0, int n1, int n2) {
+  constexpr int G = kArriveGroups / kGroupBlocks;  // groups, and warps, of a block
+  static_assert(kSumThreads == 32 * G, "a thread per lane and group");
+  __shared__ double sh[32][G + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = blockIdx.y;
+  const int g = threadIdx.x % G, l = threadIdx.x / G;
+  if (*(volatile int*)&f.a.st->done) return;
+  const double* P = q == 0 ? f.a.P0 : q == 1 ? f.a.P1 : f.a.P2;
+  const int n = q == 0 ? n0 : q == 1 ? n1 : n2;
+  constexpr int U = 8, kRound = 32 * kArriveGroups;
+  double acc = 0.0;
+  for (int i = blockIdx.x * G + g + kArriveGroups * l; i < n; i += U * kRound) {
+    double v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = i + u * kRound < n ? __ldcg(P + i + u * kRound) : 0.0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) acc += v[u];
+  }
+  sh[l][g] = acc;
+  __syncthreads();
+  const double s = warp_sum(sh[lane][warp]);
+  if (lane == 0) __stcg(&f.a.st->gpart[q][blockIdx.x * G + warp], s);
+}
+
 // alpha = delta / d^T q from n partials in every thread of the block (all of them call);
 // block 0 records it.
 __device__ __forceinline__ double block_alpha(const PcgArgs& a, const MapDesc& M, MapState* S, const double* P, int n) {
@@ -142,8 +172,10 @@ __device__ __forceinline__ double block_alpha(const PcgArgs& a, const MapDesc& M
 // mixed form's per-block arrays.  Then the WHILE
 // loop's guard: a map that has stopped -- or was never active in this outer pass -- clears the
 // condition, and so does a loop that has run past l_max (reported as a time-out).
+// groups: k_f_groups has been there, and its sums take the partials' place (one to a group, so
+// the rest of the sum is the same).
 __global__ void __launch_bounds__(3 * kSumThreads) k_f_finish(const __grid_constant__ FcgArgs f, int ph, int n0, int n1, int n2,
-                                                              int blocks) {
+                                                              int blocks, int groups) {
   __shared__ double part[3][kArriveGroups];
   __shared__ double sum[3];
   MapState* S = f.a.st;
@@ -153,8 +185,8 @@ __global__ void __launch_bounds__(3 * kSumThreads) k_f_finish(const __grid_const
   const ScalarIn in = threadIdx.x == 0 ? load_scalars(S) : ScalarIn{};
   if (!done) {
     const int q = threadIdx.x / kSumThreads, r = threadIdx.x % kSumThreads;
-    const double* P = (blocks >> q & 1) ? block_part(a, q) : q == 0 ? a.P0 : q == 1 ? a.P1 : a.P2;
-    group_sums(P, q == 0 ? n0 : q == 1 ? n1 : n2, r, part[q]);
+    const double* P = groups ? S->gpart[q] : (blocks >> q & 1) ? block_part(a, q) : q == 0 ? a.P0 : q == 1 ? a.P1 : a.P2;
+    group_sums(P, groups ? kArriveGroups : q == 0 ? n0 : q == 1 ? n1 : n2, r, part[q]);
     __syncthreads();
     if (r < 32) {
       const double v = warp_sum(part[q][r]);
@@ -162,7 +194,7 @@ __global__ void __launch_bounds__(3 * kSumThreads) k_f_finish(const __grid_const
     }
     __syncthreads();
   }
-  if (threadIdx.x != 0) return;
+  if (threadIdx.x != 0 || (done && (blockIdx.x | blockIdx.y))) return;
   if (!done && finish_scalars(a, M, S, in, ph, sum[0], sum[1], sum[2])) {
     done = 1;
     S->done = 1;
@@ -235,7 +267,8 @@ __device__ __forceinline__ void cpa16f(void* sdst, const void* gsrc) {
 }
 
 // alpha; phi += alpha d; r -= alpha q and r^T s_k (not on refresh iterations).  One tile per warp.
-__global__ void __launch_bounds__(kThreads) k_f_b(const __grid_constant__ FcgArgs f) {
+// groups: d^T q as k_f_groups' group sums instead of tile partials.
+__global__ void __launch_bounds__(kThreads) k_f_b(const __grid_constant__ FcgArgs f, int groups) {
   extern __shared__ __align__(16) unsigned char fb_dsm[];
   const PcgArgs& a = f.a;
   const int lane = threadIdx.x & 31;
@@ -270,7 +303,7 @@ __global__ void __launch_bounds__(kThreads) k_f_b(const __grid_constant__ FcgArg
     if (have && !refresh && g.i0 + k < g.i1) issue(ring[k], g.i0 + k);
     cpa_commit();
   }
-  const double alpha = block_alpha(a, M, S, a.P0 + M.tile_base, M.ntiles);
+  const double alpha = block_alpha(a, M, S, groups ? S->gpart[0] : a.P0, groups ? kArriveGroups : M.ntiles);
   if (!have) return;
   if (refresh) {
     // phi only: rows in groups of four, all loads of a group first
@@ -686,15 +719,35 @@ static cudaError_t fcg_precond(Plan& pl, int kind, const FcgArgs& f, cudaStream_
 // D rides on the multigrid cycle's last kernel where the plan allows it
 static bool fused_dots(const Plan& pl, int kind) { return kind == ULP_PRECOND_MG && mg_fuses_dots(*pl.mg); }
 
+// FP64 solves of many tiles (a small tile_rows, or maps past the size where the plan's tiles
+// reach 64 rows) add the tile partials up once, in kernels of a few blocks, instead of in every
+// block of phase B and in one block at the end.  ms a call, every block / once / with the sums
+// counted in by the tiles: multigrid 2048x2048, 30 iterations, tile_rows 4 (16384 tiles) 12.67 /
+// 10.22 / 10.24, tile_rows 8 10.24 / 9.44 / 9.58, tile_rows 2 20.8 / 12.3 / 12.0; 8192x8192, 20
+// iterations (16384 tiles) 63.5 / 61.7 / 64.2; red-black SSOR 2048x2048, tile_rows 4, 21.0 / 18.5
+// / 19.0.  The line is at four rounds of a block's sum: at 4096 tiles (4096x4096) 18.03 / 18.14 /
+// 18.67, at 2432 (2048x2048) and below the launches cost as much as they save.
+constexpr int kManyTiles = 4 * 32 * kArriveGroups;
+static bool many_tiles(const Plan& pl, int kind, const FcgArgs& f) {
+  return !mixed_fcg(pl, kind) && f.a.ntiles > kManyTiles;
+}
+// d^T q of a solve of many tiles, and phase B.
+static void fcg_phase_b(const Plan& pl, int kind, const FcgArgs& f, cudaStream_t st) {
+  const bool groups = many_tiles(pl, kind, f);
+  if (groups) k_f_groups<<<kGroupBlocks, kSumThreads, 0, st>>>(f, f.a.ntiles, 0, 0);
+  k_f_b<<<tile_blocks(f), kThreads, kRingFSmem, st>>>(f, groups);
+}
+
 // The scalars after the start (init) or a body's dot phase.
 static void fcg_finish(Plan& pl, int kind, const FcgArgs& f, bool fd, bool init, cudaStream_t st) {
   const bool x = mixed_fcg(pl, kind);
   const int nb = tile_blocks(f), nt = f.a.ntiles, nu = fd ? mg_dot_units(*pl.mg) : nt;
   // r^T r comes from the dot phase's kernel, but in the fused mixed form from those that wrote
   // r; the third sum from phase B, the residual, or k_f_dots / k_x_dots at the start
-  const bool b1 = x && fd, b2 = x && (fd || !init);
+  const bool b1 = x && fd, b2 = x && (fd || !init), groups = many_tiles(pl, kind, f);
+  if (groups) k_f_groups<<<dim3(kGroupBlocks, 3), kSumThreads, 0, st>>>(f, nu, nu, nt);
   k_f_finish<<<1, 3 * kSumThreads, 0, st>>>(f, init ? kPhResInit : kPhFcg, nu, b1 ? nb : nu, b2 ? nb : nt,
-                                            (b1 ? 2 : 0) | (b2 ? 4 : 0));
+                                            (b1 ? 2 : 0) | (b2 ? 4 : 0), groups);
 }
 
 // Start of a solve: r = b - A phi (and its BF16 copy), the mask bits, s = M^-1 r, delta_0.
@@ -742,7 +795,7 @@ static cudaError_t fcg_iteration(Plan& pl, int kind, const FcgArgs& f, cudaStrea
     return e == cudaSuccess ? cudaGetLastError() : e;
   }
   k_f_a<<<nb, kThreads, 0, st>>>(f);
-  k_f_b<<<nb, kThreads, kRingFSmem, st>>>(f);
+  fcg_phase_b(pl, kind, f, st);
   k_f_res<<<nb, kThreads, 0, st>>>(f, 1);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = fcg_precond(pl, kind, f, st, fd);
@@ -902,7 +955,7 @@ static cudaError_t fcg_eager(Plan& pl, int kind, const FcgArgs& f, cudaStream_t 
     phase_mark(pl, st, -1);
     k_f_a<<<nb, kThreads, 0, st>>>(f);
     phase_mark(pl, st, 0);
-    k_f_b<<<nb, kThreads, kRingFSmem, st>>>(f);
+    fcg_phase_b(pl, kind, f, st);
     phase_mark(pl, st, 1);
     k_f_res<<<nb, kThreads, 0, st>>>(f, 1);
     phase_mark(pl, st, 2);
