@@ -815,7 +815,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32) k_mg_down_w(Grid f, Grid c, i
 
 // one slot of the up walker's ring: U, V, D^-1, b, x of row r, the coarse x of its
 // aggregates, and on the map's grid the mask and, in the FP64 form, r of row r - 2.  Without
-// that r a block's ring is 47 KB instead of 63 and four blocks fit an SM instead of three.
+// that r a block's ring is 47 KB instead of 63.
 struct UpSlotBase {
   float4 U[32], V[32], D[32], B[32], X[32];
   float2 XC[32];
@@ -1325,20 +1325,16 @@ MgPlan* mg_create(const MapDesc& M, void* mem, int nsm, int ntiles, int max_unit
     cudaFuncSetAttribute(k_mg_up_w<kUp32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpRingSmem<kUp32>);
   }
   // one resident wave of each walker: more warps than that run as a second, mostly idle wave.
-  // The mixed form's map grid takes the four blocks per SM that its smaller ring allows where
-  // that leaves bands of kTallBand rows at least (a band reads four rows of halo): at
-  // 4096x4096 59 rows instead of 79, 87 -> 81 us; at 2048x2048 16 rows instead of 21 measured
-  // 26.3 us against 25.6.
-  int occ_down = 0, occ_up = 0, occ_up32 = 0;
+  // The mixed form's smaller ring would allow the map grid four blocks per SM instead of three,
+  // with shorter bands (each reads four rows of halo); whole calls of 20 iterations, three /
+  // four: 2048x2048 3.74 / 3.78 ms, 3000x3000 6.61 / 6.64, 3500x3500 8.34 / 8.39, 4096x4096
+  // 10.69 / 10.78, 6000x6000 20.77 / 20.81, 8192x8192 36.81 / 36.93.
+  int occ_down = 0, occ_up = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_down, k_mg_down_w, kWalkWarps * 32, kDownRingSmem);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_up, k_mg_up_w<kUp64>, kWalkWarps * 32, kUpRingSmem<kUp64>);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_up32, k_mg_up_w<kUp32>, kWalkWarps * 32, kUpRingSmem<kUp32>);
   const long long wave_down = (long long)(occ_down > 0 ? occ_down : 1) * kWalkWarps * nsm;
   const long long wave_up = (long long)(occ_up > 0 ? occ_up : 1) * kWalkWarps * nsm;
-  const long long wave_up32 = (long long)(occ_up32 > 0 ? occ_up32 : 1) * kWalkWarps * nsm;
-  constexpr int kTallBand = 32;
-  long long wave_map = wave_up < ntiles ? wave_up : ntiles;
-  if (mixed && wave_up32 <= max_units && walk_rows(M.H, M.W, 2, wave_up32) >= kTallBand) wave_map = wave_up32;
+  const long long wave_map = wave_up < ntiles ? wave_up : ntiles;
   // walkers where even two-row bands fill a wave, tiles on the smaller grids (see the
   // walker section for the measurements)
   const long long wave = wave_up < wave_down ? wave_up : wave_down;
