@@ -105,7 +105,8 @@ typedef struct ulp_options {
   double omega;           /* SSOR relaxation in (0, 2), default 1 */
   int precision;          /* ulp_precision, default ULP_PRECISION_FP64 */
   int phi0_mode;          /* ulp_phi0_mode, default ULP_PHI0_ZERO */
-  int tile_rows;          /* rows per warp tile; 0 = autotuned table */
+  int tile_rows;          /* rows per warp tile; 0 = autotuned table (mixed-precision multigrid takes tiles of
+                             its own on maps of more tiles than run at once) */
   int blocks_per_sm;      /* resident blocks per SM of the persistent solver; 0 = autotuned */
   double spin_timeout_s;  /* bound on any in-kernel wait, default 2.0 s */
   int profile;            /* 1: record CUDA events around every persistent solver launch (ulp_plan_counters);
@@ -215,7 +216,16 @@ typedef struct ulp_map {
  * CG of ulp_unwrap on its own plan, the maps spread over eight streams (largest
  * first, on the least-loaded stream), all forked from and joined back into
  * cuda_stream.  per_map: host array of n stats or NULL (same synchronisation
- * rule as ulp_unwrap).  Returns the worst status over the maps. */
+ * rule as ulp_unwrap).  Returns the worst status over the maps.
+ *
+ * Reproducibility: a call gives the same bits every time it is made on one kind
+ * of GPU.  A map's sums are added up tile by tile, so another tile_rows (the
+ * default depends on the batch) changes last bits.  With the same tile_rows a
+ * map gives the same bits alone, in any batch and with any blocks_per_sm, except
+ * in the solvers that keep small maps on the chip (I and Jacobi, where the call's
+ * maps fit and tile_rows is at most 4 in FP64, 8 in mixed precision): they group
+ * a map's sums by where its tiles fall among the SMs, which in FP64 moves results
+ * by some 1e-13 relative.  tile_rows > 8 keeps a call off them. */
 ULP_API int ulp_unwrap_batched(ulp_plan plan, const ulp_map* maps, int precond, double tol,
                        int max_outer, int max_inner, void* cuda_stream, ulp_stats* per_map);
 

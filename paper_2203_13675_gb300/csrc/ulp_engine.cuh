@@ -311,7 +311,6 @@ __device__ __forceinline__ bool finish_scalars(const PcgArgs& a, const MapDesc& 
 // Runs in the warp whose tile arrival completed phase `ph` for map m: reduces
 // the map's tile partials in a fixed order and advances its scalars
 // (alpha = delta_new / d^T q; delta_old, delta_new, beta; stop tests).
-// ngroups: how many group sums the arrival left (0: as many as the map's tiles make).
 // The finisher is the serial tail of its kernel (every other warp has left), so it is
 // built as few dependent memory round trips as possible: lane 0 loads every field of
 // the map's state it reads in the same round of L2 loads as the group sums (only the
@@ -320,13 +319,12 @@ __device__ __forceinline__ bool finish_scalars(const PcgArgs& a, const MapDesc& 
 // kernel boundary or after the grid barrier that follows every phase of the persistent
 // kernels (whose leading __syncthreads and fence cover this warp's stores).
 static_assert(kArriveGroups <= 32, "one lane per arrival group");
-__device__ __forceinline__ void finish_map(const PcgArgs& a, const MapDesc& M, MapState* Sp, int ph, int lane,
-                                           int ngroups = 0) {
+__device__ __forceinline__ void finish_map(const PcgArgs& a, const MapDesc& M, MapState* Sp, int ph, int lane) {
   volatile MapState* S = Sp;
   // the per-group sums in group order, then a fixed shuffle tree
   const int n = M.ntiles;
-  const int ng = ngroups > 0 ? ngroups : (n < kArriveGroups ? n : kArriveGroups);
-  const int cnt = (ph == kPhA) ? 1 : (ph == kPhResInit || ph == kPhFcg) ? 3 : 2;
+  const int ng = n < kArriveGroups ? n : kArriveGroups;
+  const int cnt = (ph == kPhA) ? 1 : (ph == kPhResInit) ? 3 : 2;
   const bool own = lane < ng;
   // L2 loads: another warp wrote them, and this SM's L1 may hold an older phase's values
   double v0 = own ? __ldcg(&Sp->gpart[0][lane]) : 0.0;
@@ -384,7 +382,7 @@ __device__ __forceinline__ void tile_arrive(const PcgArgs& a, const MapDesc& M, 
   if (lane == 0) {
     __stcg(a.P0 + t, v0);
     if (ph != kPhA) __stcg(a.P1 + t, v1);
-    if (ph == kPhResInit) __stcg(a.P2 + t, v2);  // kPhFcg: P2 holds r_{k+1}^T s_k from phase B
+    if (ph == kPhResInit) __stcg(a.P2 + t, v2);
     glast = atom_add_acq_rel(&S->arrive_grp[g], 1u) == (unsigned)gsize - 1u;
   }
   glast = __shfl_sync(kFull, glast, 0);
@@ -392,7 +390,7 @@ __device__ __forceinline__ void tile_arrive(const PcgArgs& a, const MapDesc& M, 
   // the group's last tile sums the group's partials (tiles base + g + 32 m, m in order of
   // lanes then of the stride loop, then a fixed shuffle tree) in parallel with the other groups
   __syncwarp();
-  const int cnt = (ph == kPhA) ? 1 : (ph == kPhResInit || ph == kPhFcg) ? 3 : 2;
+  const int cnt = (ph == kPhA) ? 1 : (ph == kPhResInit) ? 3 : 2;
   double s0 = 0.0, s1 = 0.0, s2 = 0.0;
 #pragma unroll 4
   for (int m = lane; m < gsize; m += 32) {
@@ -424,7 +422,7 @@ __device__ __forceinline__ void tile_arrive(const PcgArgs& a, const MapDesc& M, 
 // group in order and the lanes add up as a shuffle-down tree (16, 8, 4, 2, 1) -- tile_arrive's
 // order, so both give the same bits.  A thread holds lanes c, c + 4, ..., c + 28 of its group:
 // the tree's first three levels stay in registers, where an FP64 add of a warp costs its 64
-// cycles for 32 useful lanes instead of for a few.  get(i, v): loads v[q] = partial i + 128 q.
+// cycles for 32 useful lanes instead of for a few.
 struct GroupLane {
   int g, c;
   __device__ __forceinline__ explicit GroupLane(int r) : g(((r >> 5) << 3) + (r & 7)), c((r & 31) >> 3) {}

@@ -1,21 +1,22 @@
-// ulp_fcg.cu -- inner solve with the DCT Poisson preconditioner: flexible CG in
-// one CUDA graph.
+// ulp_fcg.cu -- inner solve with the preconditioners that are kernels of their own (DCT,
+// multigrid, red-black, learned): flexible CG in one CUDA graph.
 //
-// The DCT preconditioner runs on the tensor cores as four GEMM launches, so
-// this solve is not a single persistent kernel: each phase of an iteration is
-// its own kernel and the loop is a graph WHILE node whose condition the
-// device clears when the map stops (converged, l_max or breakdown), so the
-// host never waits inside the solve.  The BF16 GEMMs make M^-1 slightly
+// Each phase of an iteration is its own kernel and the loop is a graph WHILE node
+// whose condition the device clears when the map stops (converged, l_max or
+// breakdown), so the host never waits inside the solve.  The kernels leave partials
+// of their dot products; phase B adds those of d^T q for its alpha, and k_f_finish
+// at the end of an iteration the others.  The DCT's BF16 GEMMs, for one, make M^-1 slightly
 // inexact and not exactly symmetric, so beta is the flexible (Polak-Ribiere)
 // one, beta = r_{k+1}^T (s_{k+1} - s_k) / r_k^T s_k; the term r_{k+1}^T s_k is
 // accumulated in phase B, before the GEMMs overwrite s.  All vectors, alpha,
 // beta and the stop tests are FP64, as in the other FP64 solvers.
 //
-// Per iteration:  A: d = s + beta d, q = A d, d^T q -> alpha
-//                 B: phi += alpha d, r -= alpha q (not on refresh iterations), r^T s_k
-//                 R: on refresh iterations r = b - A phi, r^T s_k
-//                 DCT: s = Pi L^+ r (4 tcgen05 GEMMs on the BF16 copy of r that B and R write)
-//                 D: r^T s, r^T r -> beta, stop test, WHILE condition
+// Per iteration:  A: d = s + beta d, q = A d, partials of d^T q
+//                 B: alpha; phi += alpha d, r -= alpha q (not on refresh iterations), partials of r^T s_k
+//                 R: on refresh iterations r = b - A phi, partials of r^T s_k
+//                 M: s = M^-1 r (DCT: 4 tcgen05 GEMMs on the BF16 copy of r that B and R write)
+//                 D: partials of r^T s, r^T r (in multigrid's last kernel where it can carry them)
+//                 k_f_finish: the sums, beta, stop test, WHILE condition
 #include <cuda_bf16.h>
 
 #include "ulp_mixed.cuh"
@@ -87,9 +88,10 @@ __device__ __forceinline__ void put_rbf(const PcgArgs& a, const MapDesc& M, int 
 // SMs active for 46,000 of k_x_a's 62,800 cycles and of the last cycle kernel's 67,000).
 // Mixed multigrid, us a call, before / after, with the set-up kernels' cheaper FP64 work:
 // 256x256 1825 / 1626, 2048x2048 11062 / 10376; twelve uneven maps 18677 / 17410.
-// The mixed form, whose iterates do not depend on how the sums are grouped (its scalars are
-// rounded to FP32), makes one partial per block instead of per tile: one SM adds 512 FP64
-// values in 0.4 us, the 4096 tiles of a 4096x4096 map in 3.
+// The mixed form makes one partial per block instead of per tile: one SM adds 512 FP64 values
+// in 0.4 us, the 4096 tiles of a 4096x4096 map in 3.  Its alpha and beta are rounded to FP32, so
+// another grouping of a sum rarely changes an iterate (the same bits in every case measured); a
+// last bit can still flip such a rounding, or a stop test, which reads the FP64 sums.
 constexpr int kSumThreads = 128;  // threads that add one array of partials
 
 // The mixed form's partials per block (the persistent solvers' slots, idle here): q = 0 d^T q,
@@ -980,8 +982,10 @@ static cudaError_t fcg_eager(Plan& pl, int kind, const FcgArgs& f, cudaStream_t 
 // plan's tiles reach their 64 rows and become more than a wave.  Beyond it the mixed form,
 // whose sums are per block, takes one wave of three blocks per SM (k_x_a and k_x_b are built
 // for that): at 4096x4096 72 rows, 456 blocks, k_x_a 102 -> 82 us and k_x_b 86 -> 83 (the
-// plan's 4096 tiles are 512 blocks).  At 2048x2048 three blocks per SM, 18 rows instead of
-// 27, measured slower (k_x_a 23.9 us against 22.7).
+// plan's 4096 tiles are 512 blocks).  Whole calls of 20 iterations, the plan's tiles / these, ms:
+// 1000x5120 (2480 tiles) 4.60 / 4.42, 2500x2100 4.72 / 4.50, 3000x3000 7.15 / 6.61, 4096x4096
+// 11.11 / 10.78, 6000x6000 20.99 / 20.81, 8192x8192 36.88 / 36.93; within one wave they lose:
+// 5120x1000 (2400 tiles) 4.61 / 4.69, 2048x2048 3.74 / 3.81, 1500x1500 2.70 / 2.78.
 constexpr int kXBlocksPerSm = 3;
 int fcg_mixed_rows(int H, int nsx, int nsm) {
   const long long warps = (long long)nsm * kXBlocksPerSm * kWarps;

@@ -230,7 +230,7 @@ __device__ __forceinline__ double wrap_pv(double x) {
   const double two_pi = 2.0 * pi;
   const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
   if (h < 0x400921FBu) return __dadd_rn(x, 0.0);  // |x| < pi - 6e-7: ceil = -0
-  if (h > 0x400921FBu && h < 0x4022D97Cu)          // pi + 3e-7 < |x| < 3 pi - 3e-6: ceil = +-1
+  if (h > 0x400921FBu && h < 0x4022D97Cu)          // pi + 1.2e-6 < |x| < 3 pi - 3.7e-6: ceil = +-1
     return x > 0.0 ? __dsub_rn(x, two_pi) : __dadd_rn(x, two_pi);
   double k = ceil(__ddiv_rn(__dsub_rn(x, pi), two_pi));
   return __dsub_rn(x, __dmul_rn(two_pi, k));

@@ -519,14 +519,15 @@ __global__ void __launch_bounds__(kTileThreads) k_mg_down_t(Grid f, Grid c, int 
 
 // prolongation + correction + both post-sweeps for the rows [TR band, TR band + TR).
 // xc: the coarse grid's corrected solution.  MODE kUpCoarse: s to the grid's t plane.
-// kUp64 (the map's grid): s in FP64; with dp0, r^T s and r^T r (r: the map's FP64
-// residual) over the block's pixels arrive in the flexible CG's dot phase.  kUp32 (the
-// map's grid, mixed flexible CG): s in FP32 into s32; with dp0, the same dot phase in
-// double-float sums of exact FP32 products, r being the cycle's right-hand side.
+// kUp64 (the map's grid): s in FP64; with dp0, the partials of r^T s and r^T r (r: the map's
+// FP64 residual) over the block's pixels are left in dp0 and dp1 for the flexible CG's
+// k_f_finish.  kUp32 (the map's grid, mixed flexible CG): s in FP32 into s32; with dp0, the
+// partials of r^T s in double-float sums of exact FP32 products, r being the cycle's
+// right-hand side.
 enum { kUpCoarse = 0, kUp64 = 1, kUp32 = 2 };
 // FP64 of a lane's four values, 0 on masked pixels.  By integer instructions where all four are
 // plain numbers: a conversion holds an FP64 pipe slot, of which the FP64 form's up step is short.
-// 1251 x 937 in FP64, whole solve: 8063 us without the shortened set-up and this, 7909 us with both.
+// One solve of 40 iterations in FP64, conversions / this: 937x1251 5.24 / 5.20 ms, 2048x2048 10.78 / 10.72.
 __device__ __forceinline__ void widen_masked(const float4& v, const uchar4& mk, double (&s)[4]) {
   if (is_plain(v.x) && is_plain(v.y) && is_plain(v.z) && is_plain(v.w)) {
     s[0] = mk.x ? 0.0 : widen_plain(v.x);
@@ -940,13 +941,13 @@ __global__ void __launch_bounds__(kWalkWarps * 32) k_mg_up_w(Grid f, Grid c, con
             if (rv) {
               const double2 ra = sl.RA[lane], rb2 = sl.RB[lane];
               const double rk[4] = {ra.x, ra.y, rb2.x, rb2.y};
-  #pragma unroll
+#pragma unroll
               for (int k = 0; k < 4; ++k)
                 if (j + k < f.W) {
                   rs = fma(rk[k], sv[k], rs);
                   rr = fma(rk[k], rk[k], rr);
                 }
-          }
+            }
           }
         }
       }

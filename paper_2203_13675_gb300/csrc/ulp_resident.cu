@@ -5,8 +5,8 @@
 // Same tiles and the same arithmetic per pixel as k_pcg64 / k_pcg32.  There a phase streams
 // its planes from L2 a row at a time, and with one or two warps per SM partition each row
 // costs its load latency: at 640x480 the FP64 pipe (64 cycles per warp instruction and
-// partition; about 70 of them per tile in phase A, 50 in phase B) was busy for 15,000 of
-// 62,000 cycles of an iteration.  Here a warp keeps its tile's weights, D, D^-1, phi (or
+// partition; about 70 of them per tile in phase A, 50 in phase B) was busy for a quarter of
+// an iteration.  Here a warp keeps its tile's weights, D, D^-1, phi (or
 // the correction), r and s in shared memory and d and q in registers across iterations.
 // What crosses tiles is the rim of s: in phase B a warp stores its first and last row and
 // its two edge columns into the map's s plane (r for M = I), and in phase A it reads its
@@ -24,9 +24,16 @@
 // Measured on one GB300, us per Jacobi iteration (tile partials, finisher warp and grid
 // barriers / here): FP64 256x256 33.4 / 11.8, 640x480 33.0 / 14.9, 704x704 37.7 / 23.5; mixed
 // 256x256 26.3 / 10.7, 1024x1024 34.5 / 20.4, 1200x1024 36.4 / 21.7.  The streaming kernels
-// with published partials take 27.8 at 640x480 (FP64) and 32.8 at 1024x1024 (mixed).  Of the
-// 31,600 cycles of an iteration at 640x480, 15,700 are the two tile phases, 5,300 the
-// blocks' sums and fences, 6,800 the trips through L2, 2,800 the scalars.
+// with published partials take 27.8 at 640x480 (FP64) and 32.8 at 1024x1024 (mixed).  Clock
+// stamps in a build made for it put half of an iteration at 640x480 into the two tile phases, a
+// sixth into the blocks' sums and fences, a fifth into the trips through L2 and a tenth into
+// the scalars.
+//
+// A map's sums are grouped by where its tiles fall among the blocks, so its last bits depend on
+// the batch and the number of SMs (the streaming kernels' do not).  One partial per tile in the
+// streaming kernels' order instead gives their bits and was measured at 0.87-0.95 of the speed
+// in FP64, 0.77-0.93 in mixed precision: every SM then adds all of the map's tile partials at
+// 64 cycles per warp of FP64 values, and polls as many lines.
 #include <type_traits>
 
 #include "ulp_flow32.cuh"
