@@ -269,8 +269,9 @@ __device__ __forceinline__ void cpa16f(void* sdst, const void* gsrc) {
 }
 
 // alpha; phi += alpha d; r -= alpha q and r^T s_k (not on refresh iterations).  One tile per warp.
-// groups: d^T q as k_f_groups' group sums instead of tile partials.
-__global__ void __launch_bounds__(kThreads) k_f_b(const __grid_constant__ FcgArgs f, int groups) {
+// GROUPS: d^T q as k_f_groups' group sums instead of tile partials.
+template <bool GROUPS>
+__global__ void __launch_bounds__(kThreads) k_f_b(const __grid_constant__ FcgArgs f) {
   extern __shared__ __align__(16) unsigned char fb_dsm[];
   const PcgArgs& a = f.a;
   const int lane = threadIdx.x & 31;
@@ -305,7 +306,7 @@ __global__ void __launch_bounds__(kThreads) k_f_b(const __grid_constant__ FcgArg
     if (have && !refresh && g.i0 + k < g.i1) issue(ring[k], g.i0 + k);
     cpa_commit();
   }
-  const double alpha = block_alpha(a, M, S, groups ? S->gpart[0] : a.P0, groups ? kArriveGroups : M.ntiles);
+  const double alpha = block_alpha(a, M, S, GROUPS ? S->gpart[0] : a.P0 + M.tile_base, GROUPS ? kArriveGroups : M.ntiles);
   if (!have) return;
   if (refresh) {
     // phi only: rows in groups of four, all loads of a group first
@@ -735,9 +736,12 @@ static bool many_tiles(const Plan& pl, int kind, const FcgArgs& f) {
 }
 // d^T q of a solve of many tiles, and phase B.
 static void fcg_phase_b(const Plan& pl, int kind, const FcgArgs& f, cudaStream_t st) {
-  const bool groups = many_tiles(pl, kind, f);
-  if (groups) k_f_groups<<<kGroupBlocks, kSumThreads, 0, st>>>(f, f.a.ntiles, 0, 0);
-  k_f_b<<<tile_blocks(f), kThreads, kRingFSmem, st>>>(f, groups);
+  if (many_tiles(pl, kind, f)) {
+    k_f_groups<<<kGroupBlocks, kSumThreads, 0, st>>>(f, f.a.ntiles, 0, 0);
+    k_f_b<true><<<tile_blocks(f), kThreads, kRingFSmem, st>>>(f);
+  } else {
+    k_f_b<false><<<tile_blocks(f), kThreads, kRingFSmem, st>>>(f);
+  }
 }
 
 // The scalars after the start (init) or a body's dot phase.
@@ -808,7 +812,9 @@ static cudaError_t fcg_iteration(Plan& pl, int kind, const FcgArgs& f, cudaStrea
 
 // Dynamic shared memory above 48 KB is an attribute of the function on the current device.
 static cudaError_t fcg_attrs() {
-  const cudaError_t e = cudaFuncSetAttribute(k_f_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingFSmem);
+  cudaError_t e = cudaFuncSetAttribute(k_f_b<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingFSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_f_b<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingFSmem);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_x_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingBSmem);
 }
